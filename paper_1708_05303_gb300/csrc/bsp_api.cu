@@ -22,7 +22,7 @@ using namespace bsp;
 namespace {
 
 thread_local std::string g_last_error;
-constexpr int CCOLS = 64;   // pairs per CUDA-core contraction tile (bsp_contract.cu)
+constexpr int CCOLS = 64;   // columns of a CUDA-core contraction slot (bsp_contract.cu)
 
 bsp_status cuda_fail(cudaError_t e, const char* where) {
     g_last_error = std::string(where) + ": " + cudaGetErrorString(e);
@@ -193,6 +193,141 @@ bsp_status upload_sched(DevSched& d, const HostSched& h) {
 
 size_t partial_bytes(const HostSched& h, int cols) {
     return (size_t)h.works.size() * h.nsplit * 64 * cols * sizeof(double);
+}
+
+// FP32 contraction schedule (k_contract_oct).  The pairs (b, c) come in octets
+// (b; c = 8 j .. 8 j + 7); an octet's rows are (l, a) for a in its own a-range.
+// Sorted by the length of that range, the 16 octets of a work waste few rows
+// (32 shells, l = 0, 2, 4: 20 480 multiply-adds per point for 10 872 useful).  All
+// warps of a work run the same number of rows: letting each warp have its own put
+// the long ones on one SM partition, and several unrolled variants side by side
+// missed the instruction cache (32 against 21 ms per contraction at 256^3).  A row
+// list longer than a thread's rows takes several works.
+struct OctSched {
+    std::vector<OctWork> works;
+    std::vector<int> stage;
+    std::vector<BinLoc> loc;   // [out_slots][nbins]
+    int nsplit = 1, max_a = 0, max_x = 0;
+};
+
+struct DevOct {
+    OctWork* works = nullptr;
+    int* stage = nullptr;
+    BinLoc* loc = nullptr;
+    void release() {
+        cudaFree(works); cudaFree(stage); cudaFree(loc);
+        works = nullptr; stage = nullptr; loc = nullptr;
+    }
+};
+
+OctSched build_oct_sched(const BinList& bins, const std::vector<int>& out_slots, int nsh, size_t npts,
+                         int target_ctas, int nsm) {
+    OctSched h;
+    struct Oct { int j, b, alo, ahi; };
+    std::vector<int> at(64 * 8, -1);   // (b, j) -> octet
+    std::vector<Oct> oct;
+    for (auto& t : bins) {
+        int& k = at[t[1] * 8 + t[2] / 8];
+        if (k < 0) {
+            k = (int)oct.size();
+            oct.push_back(Oct{t[2] / 8, t[1], t[0], t[0]});
+        }
+        oct[k].alo = std::min(oct[k].alo, t[0]);
+        oct[k].ahi = std::max(oct[k].ahi, t[0]);
+    }
+    std::vector<int> order(oct.size());
+    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
+    std::sort(order.begin(), order.end(), [&](int x, int y) {
+        const Oct &u = oct[x], &v = oct[y];
+        return std::make_tuple(u.alo - u.ahi, u.j, u.b) < std::make_tuple(v.alo - v.ahi, v.j, v.b);
+    });
+    struct Place { int work0, per, len, slot; };
+    std::vector<Place> place(oct.size());
+    const int ne = (int)out_slots.size();
+    for (size_t o0 = 0; o0 < order.size(); o0 += OCT_SLOTS) {
+        const int ns = (int)std::min<size_t>(OCT_SLOTS, order.size() - o0);
+        auto octet = [&](int k) -> const Oct& { return oct[order[o0 + std::min(k, ns - 1)]]; };   // empty slots: the last one
+        int len = 0;
+        for (int k = 0; k < ns; ++k) len = std::max(len, octet(k).ahi - octet(k).alo + 1);
+        const int blocks = (len * ne + 7) / 8;   // row blocks of 8, shared evenly by the works they take
+        const int nch = (blocks + OCT_TRMAX - 1) / OCT_TRMAX, tr = (blocks + nch - 1) / nch;
+        // the pair factors: each octet's eight shells in a row (past the last shell: repeated), then the other b
+        std::vector<int> xs;
+        int crow[OCT_SLOTS], brow[OCT_SLOTS];
+        for (int k = 0; k < OCT_SLOTS; ++k) {
+            crow[k] = -1;
+            for (int q = 0; q < k; ++q)
+                if (octet(q).j == octet(k).j) crow[k] = crow[q];
+            if (crow[k] >= 0) continue;
+            crow[k] = (int)xs.size();
+            for (int c = 0; c < 8; ++c) xs.push_back(std::min(8 * octet(k).j + c, nsh - 1));
+        }
+        for (int k = 0; k < OCT_SLOTS; ++k) {
+            const int b = octet(k).b;
+            brow[k] = (int)(std::find(xs.begin(), xs.end(), b) - xs.begin());
+            if (brow[k] == (int)xs.size()) xs.push_back(b);
+        }
+        const int work0 = (int)h.works.size();
+        for (int c0 = 0; c0 < nch; ++c0) {
+            OctWork w{};
+            std::vector<int> fields[OCT_SLOTS], staged;
+            w.tr = std::min(tr, blocks - tr * c0);
+            for (int k = 0; k < OCT_SLOTS; ++k) {
+                const Oct& o = octet(k);
+                w.brow[k] = brow[k];
+                w.crow[k] = crow[k];
+                for (int r = 0; r < 8 * w.tr; ++r) {
+                    const int i = 8 * tr * c0 + r, si = std::min(i / len, ne - 1);
+                    fields[k].push_back(out_slots[si] * nsh + std::min(o.alo + i % len, o.ahi));
+                }
+                staged.insert(staged.end(), fields[k].begin(), fields[k].end());
+            }
+            // staged in field order: consecutive rows of a slot are consecutive in shared memory
+            std::sort(staged.begin(), staged.end());
+            staged.erase(std::unique(staged.begin(), staged.end()), staged.end());
+            for (int k = 0; k < OCT_SLOTS; ++k)
+                for (size_t r = 0; r < fields[k].size(); ++r)
+                    w.arow[k][r] = (uint16_t)(std::lower_bound(staged.begin(), staged.end(), fields[k][r]) - staged.begin());
+            w.nA = (int)staged.size();
+            w.nX = (int)xs.size();
+            w.stage0 = (int)h.stage.size();
+            h.stage.insert(h.stage.end(), staged.begin(), staged.end());
+            h.stage.insert(h.stage.end(), xs.begin(), xs.end());
+            h.max_a = std::max(h.max_a, w.nA);
+            h.max_x = std::max(h.max_x, w.nX);
+            h.works.push_back(w);
+        }
+        for (int k = 0; k < ns; ++k) place[order[o0 + k]] = Place{work0, 8 * tr, len, k};
+    }
+    h.loc.resize(out_slots.size() * bins.size());
+    for (size_t b = 0; b < bins.size(); ++b) {
+        const int k = at[bins[b][1] * 8 + bins[b][2] / 8];
+        const Place& pl = place[k];
+        for (size_t si = 0; si < out_slots.size(); ++si) {
+            const int i = (int)si * pl.len + bins[b][0] - oct[k].alo;
+            h.loc[si * bins.size() + b] = BinLoc{pl.work0 + i / pl.per, i % pl.per, 8 * pl.slot + bins[b][2] % 8, 0};
+        }
+    }
+    const int nw = std::max<int>(1, (int)h.works.size());
+    // segments of at least 1024 points: 2 500 cycles of multiply-adds or more, against
+    // a CTA's start and its 56 x 128 partial sums; and whole waves of the three CTAs an
+    // SM holds where there is at least one (64^3: 456 CTAs instead of 512)
+    const long long by_len = (long long)((npts + 1023) / 1024), by_ctas = (target_ctas + nw - 1) / nw, wave = 3LL * nsm;
+    long long split = std::max<long long>(1, std::min(by_len, by_ctas));
+    if (split * nw >= wave) split = std::max<long long>(1, split * nw / wave * wave / nw);
+    h.nsplit = (int)split;
+    return h;
+}
+
+constexpr size_t OCT_UNIT = OCT_ROWS * OCT_COLS;   // FP64 partial values per FP32 CTA
+size_t partial_bytes(const OctSched& h) { return h.works.size() * h.nsplit * OCT_UNIT * sizeof(double); }
+
+bsp_status upload_oct(DevOct& d, const OctSched& h) {
+    d.release();
+    bsp_status s;
+    if ((s = upload(&d.works, h.works)) != BSP_OK) return s;
+    if ((s = upload(&d.stage, h.stage)) != BSP_OK) return s;
+    return upload(&d.loc, h.loc);
 }
 
 // Tensor-core schedule: tiles of <= 128 pairs (sorted by (b, c), shells
@@ -368,7 +503,7 @@ struct bsp_plan {
     std::vector<int> out_slots;  // slot of each output multipole
     int prec = 0;
     FftGeom geom{};
-    int target_ctas = 2048;
+    int target_ctas = 4096;           // FP32 contraction (4 100 CTAs against 2 050: 88 against 93 ms for shot noise on 256^3)
     int fb_cap = 1;                   // FFT batch width the workspace was sized for
     int16_t* d_shell_of = nullptr;
     FieldDesc* d_fd_raw = nullptr;    // one field: delta on every mode but the mean (skew spectrum)
@@ -387,8 +522,8 @@ struct bsp_plan {
     bool need_u = false;
     float* d_radial = nullptr;        // [n_funcs][n2max + 1]
     int* d_ells = nullptr;
-    HostSched u_sched;                // rows M0_a, pairs M2_b M2_c
-    DevSched u_dev;
+    OctSched u_sched;                 // rows M0_a, pairs M2_b M2_c
+    DevOct u_dev;
     TcSched tc_u_sched;
     TcWork* d_tcu_works = nullptr;
     int2* d_tcu_pairs = nullptr;
@@ -411,8 +546,8 @@ struct bsp_plan {
     BinList vbins;                    // valid sorted bins a >= b >= c and their counts
     std::vector<double> vcounts;
     double* d_counts = nullptr;
-    HostSched comp_sched;
-    DevSched comp_dev;
+    OctSched comp_sched;              // FP32 plans
+    DevOct comp_dev;
     // tensor-core path
     bool tc = false;
     int nprod = 3;
@@ -708,14 +843,13 @@ bsp_status bsp_plan_create(bsp_plan** out, int n, double box, int n_shells, cons
             return st;
         }
     }
-    p->cand_sched = build_sched(p->cand, std::vector<int>{0}, n_shells, p->nrep, p->target_ctas, CCOLS);
+    p->cand_sched = build_sched(p->cand, std::vector<int>{0}, n_shells, p->nrep, 2048, CCOLS);
     if ((st = upload_sched(p->cand_dev, p->cand_sched)) != BSP_OK) {
         delete p;
         return st;
     }
     // workspace sizing: compute schedule bounded by the candidate output bins
     const BinList ocand = p->full ? expand_full(p->cand) : p->cand;
-    HostSched bound = build_sched(ocand, p->out_slots, n_shells, p->npts(), p->target_ctas, CCOLS);
     size_t t1, t2;
     t12_sizes(g, sizeof(float), &t1, &t2);
     const size_t nfields32 = (size_t)p->nslot() * n_shells;
@@ -725,11 +859,16 @@ bsp_status bsp_plan_create(bsp_plan** out, int n, double box, int n_shells, cons
     t12_sizes(g, sizeof(double), &t1, &t2);
     p->fld64_bytes = round256((size_t)n_shells * p->npts() * sizeof(double));
     p->fb64 = (int)std::max<size_t>(1, std::min<size_t>(n_shells, (size_t)(2ull << 30) / (t1 + t2)));
-    // the valid-bin schedule has at most as many works as the bound, and
-    // nsplit <= ceil(target / nwork), so nwork * nsplit <= target + nwork
-    p->part_bytes = round256(std::max(partial_bytes(bound, CCOLS),
-                                      (size_t)(4096 + bound.works.size()) * 64 * CCOLS * sizeof(double)));
-    if (p->shot) p->part_bytes *= 4;   // main sum + three shot-noise sums
+    if (!p->tc) {
+        // the valid-bin schedule has at most as many works as the candidates' (a few
+        // more where its octets pack less evenly), and nsplit <= ceil(target / nwork),
+        // so nwork * nsplit <= target + nwork
+        const OctSched bound = build_oct_sched(ocand, p->out_slots, n_shells, p->npts(), p->target_ctas, p->nsm);
+        const size_t nw = bound.works.size() + 8;
+        p->part_bytes = round256((std::min<size_t>(4096, nw * ((p->npts() + 1023) / 1024)) + nw) * OCT_UNIT *
+                                 sizeof(double));
+        if (p->shot) p->part_bytes *= 4;   // main sum + three shot-noise sums
+    }
     p->tout_bytes = round256(p->ells.size() * ocand.size() * sizeof(double));
     if (p->tc) {
         p->kb_rows32 = n_shells;
@@ -860,17 +999,17 @@ bsp_status bsp_plan_create_modal(bsp_plan** out, int n, double box, int n_funcs,
     p->tfull_bytes = round256(p->ells.size() * nall * sizeof(double));
     p->ufull_bytes = p->need_u ? round256(nall * sizeof(double)) : 0;
     if (!p->tc) {
-        p->comp_sched = build_sched(p->bins, p->out_slots, nf, p->npts(), p->target_ctas, CCOLS);
+        p->comp_sched = build_oct_sched(p->bins, p->out_slots, nf, p->npts(), p->target_ctas, p->nsm);
         p->fld32_bytes = round256(nfields * p->npts() * sizeof(float));
-        p->part_bytes = round256(partial_bytes(p->comp_sched, CCOLS));
-        if ((st = upload_sched(p->comp_dev, p->comp_sched)) != BSP_OK) {
+        p->part_bytes = round256(partial_bytes(p->comp_sched));
+        if ((st = upload_oct(p->comp_dev, p->comp_sched)) != BSP_OK) {
             delete p;
             return st;
         }
         if (p->need_u) {
-            p->u_sched = build_sched(p->bins, std::vector<int>{0}, nf, p->npts(), p->target_ctas, CCOLS);
-            p->upart_bytes = round256(partial_bytes(p->u_sched, CCOLS));
-            if ((st = upload_sched(p->u_dev, p->u_sched)) != BSP_OK) {
+            p->u_sched = build_oct_sched(p->bins, std::vector<int>{0}, nf, p->npts(), p->target_ctas, p->nsm);
+            p->upart_bytes = round256(partial_bytes(p->u_sched));
+            if ((st = upload_oct(p->u_dev, p->u_sched)) != BSP_OK) {
                 delete p;
                 return st;
             }
@@ -956,11 +1095,12 @@ static void set_output_bins(bsp_plan* p) {
 }
 
 static bsp_status finish_counts(bsp_plan* p) {
-    p->comp_sched = build_sched(p->bins, p->out_slots, p->nsh, p->npts(), p->target_ctas, CCOLS);
-    if (round256(partial_bytes(p->comp_sched, CCOLS)) * (p->shot ? 4 : 1) > p->part_bytes) return BSP_ENOMEM;
-    bsp_status s = upload_sched(p->comp_dev, p->comp_sched);
-    if (s != BSP_OK) return s;
-    if (p->tc) {
+    bsp_status s;
+    if (!p->tc) {
+        p->comp_sched = build_oct_sched(p->bins, p->out_slots, p->nsh, p->npts(), p->target_ctas, p->nsm);
+        if (round256(partial_bytes(p->comp_sched)) * (p->shot ? 4 : 1) > p->part_bytes) return BSP_ENOMEM;
+        if ((s = upload_oct(p->comp_dev, p->comp_sched)) != BSP_OK) return s;
+    } else {
         p->tc_sched = build_tc_sched(p->bins, p->out_slots, p->pad16, p->npts(), p->nsm, p->tc_max_boxes);
         if (round256(p->tc_sched.units.size() * TC_UNIT * sizeof(double)) > p->tc_part_bytes) return BSP_ENOMEM;
         cudaFree(p->d_tc_works); cudaFree(p->d_tc_pairs); cudaFree(p->d_tc_loc); cudaFree(p->d_tc_units);
@@ -1004,8 +1144,8 @@ bsp_status bsp_counts(bsp_plan* p, void* ws, void* stream) {
     if (e != cudaSuccess) return cuda_fail(e, "gather (counts)");
     double* partial = (double*)(base + L.partial);
     double* cnt = (double*)(base + L.cnt);
-    e = launch_contract_cc<double>(wrows, urows, nullptr, 0, p->nrep, p->cand_dev.works, p->cand_dev.nwork,
-                                   p->cand_dev.pairs, p->cand_dev.rowf, p->nrep, p->cand_dev.nsplit, partial, st);
+    e = launch_contract_f64(wrows, urows, p->nrep, p->cand_dev.works, p->cand_dev.nwork, p->cand_dev.pairs,
+                            p->cand_dev.rowf, p->nrep, p->cand_dev.nsplit, partial, st);
     if (e != cudaSuccess) return cuda_fail(e, "contract (counts)");
     const double n3 = (double)p->npts();
     e = launch_reduce(partial, p->cand_dev.nsplit, 0, 0, p->cand_dev.loc, (int)p->cand.size(),
@@ -1151,7 +1291,7 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
     if ((ms = mark(p, st, 1)) != BSP_OK) return ms;
     double* partial = (double*)(base + L.partial);
     double* tout = (double*)(base + L.tout);
-    const size_t pstride = round256(partial_bytes(p->comp_sched, CCOLS)) / sizeof(double);
+    const size_t pstride = round256(partial_bytes(p->comp_sched)) / sizeof(double);
     const size_t fs = (size_t)nf * p->npts();
     const float* F = f32;
     const float* S = f32 + fs;
@@ -1162,10 +1302,10 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
                    {W, S, W, 1},            // rows W^l_a, pairs S_b I_c + I_b S_c
                    {W, W, nullptr, 0}};     // rows W^l_a, pairs I_b I_c
     for (int j = 0; j < (shot ? 4 : 1); ++j) {
-        cudaError_t e = launch_contract_cc<float>(jobs[j].rows, jobs[j].px, jobs[j].py, jobs[j].sym, p->npts(),
-                                                  p->comp_dev.works, p->comp_dev.nwork, p->comp_dev.pairs,
-                                                  p->comp_dev.rowf, p->npts(), p->comp_dev.nsplit,
-                                                  partial + j * pstride, st);
+        cudaError_t e = launch_contract_oct(jobs[j].rows, jobs[j].px, jobs[j].py, jobs[j].sym, p->npts(),
+                                            p->comp_dev.works, (int)p->comp_sched.works.size(), p->comp_dev.stage,
+                                            p->comp_sched.max_a, p->comp_sched.max_x, p->npts(), p->comp_sched.nsplit,
+                                            partial + j * pstride, st);
         if (e != cudaSuccess) return cuda_fail(e, "contract");
         ++launches;
     }
@@ -1182,8 +1322,8 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
         sh.coef[1] = 1.0 / (V * nbar * n3);
         sh.coef[2] = -2.0 / (nbar * nbar * n3);
     }
-    cudaError_t e = launch_reduce(partial, p->comp_dev.nsplit, 0, 0, p->comp_dev.loc, p->comp_dev.nloc,
-                                  (int)p->bins.size(), p->d_counts, 1.0 / (V * n3), 1, tout, B, st,
+    cudaError_t e = launch_reduce(partial, p->comp_sched.nsplit, OCT_UNIT, OCT_COLS, p->comp_dev.loc,
+                                  (int)p->comp_sched.loc.size(), (int)p->bins.size(), p->d_counts, 1.0 / (V * n3), 1, tout, B, st,
                                   shot ? &sh : nullptr);
     if (e != cudaSuccess) return cuda_fail(e, "reduce");
     if ((ms = mark(p, st, 3)) != BSP_OK) return ms;
@@ -1220,25 +1360,25 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
         }
         if ((ms = mark(p, st, 1)) != BSP_OK) return ms;
         double* part = (double*)(base + L.partial);
-        cudaError_t e = launch_contract_cc<float>(f32, f32, nullptr, 0, p->npts(), p->comp_dev.works,
-                                                  p->comp_dev.nwork, p->comp_dev.pairs, p->comp_dev.rowf,
-                                                  p->npts(), p->comp_dev.nsplit, part, st);
+        cudaError_t e = launch_contract_oct(f32, f32, nullptr, 0, p->npts(), p->comp_dev.works,
+                                            (int)p->comp_sched.works.size(), p->comp_dev.stage, p->comp_sched.max_a,
+                                            p->comp_sched.max_x, p->npts(), p->comp_sched.nsplit, part, st);
         if (e != cudaSuccess) return cuda_fail(e, "contract (modal)");
         ++launches;
         if (p->need_u) {
             const float* m2 = f32 + (size_t)p->slot2 * nf * p->npts();
-            e = launch_contract_cc<float>(f32, m2, nullptr, 0, p->npts(), p->u_dev.works, p->u_dev.nwork,
-                                          p->u_dev.pairs, p->u_dev.rowf, p->npts(), p->u_dev.nsplit,
-                                          part + p->part_bytes / sizeof(double), st);
+            e = launch_contract_oct(f32, m2, nullptr, 0, p->npts(), p->u_dev.works, (int)p->u_sched.works.size(),
+                                    p->u_dev.stage, p->u_sched.max_a, p->u_sched.max_x, p->npts(), p->u_sched.nsplit,
+                                    part + p->part_bytes / sizeof(double), st);
             if (e != cudaSuccess) return cuda_fail(e, "contract (modal U)");
             ++launches;
         }
         if ((ms = mark(p, st, 2)) != BSP_OK) return ms;
-        e = launch_reduce(part, p->comp_dev.nsplit, 0, 0, p->comp_dev.loc, p->comp_dev.nloc, (int)nall,
+        e = launch_reduce(part, p->comp_sched.nsplit, OCT_UNIT, OCT_COLS, p->comp_dev.loc, (int)p->comp_sched.loc.size(), (int)nall,
                           p->d_counts, 1.0, 2, nullptr, tfull, st);
         if (e == cudaSuccess && p->need_u)
-            e = launch_reduce(part + p->part_bytes / sizeof(double), p->u_dev.nsplit, 0, 0, p->u_dev.loc,
-                              p->u_dev.nloc, (int)nall, p->d_counts, 1.0, 2, nullptr, ufull, st);
+            e = launch_reduce(part + p->part_bytes / sizeof(double), p->u_sched.nsplit, OCT_UNIT, OCT_COLS, p->u_dev.loc,
+                              (int)p->u_sched.loc.size(), (int)nall, p->d_counts, 1.0, 2, nullptr, ufull, st);
         if (e != cudaSuccess) return cuda_fail(e, "reduce (modal)");
         launches += p->need_u ? 2 : 1;
     } else {
@@ -1341,8 +1481,7 @@ bsp_status bsp_plan_stats(const bsp_plan* p, double* st) {
         works = (double)p->tc_sched.works.size();
         nsplit = (double)p->tc_sched.units.size();
     } else {
-        // 64 pairs times the 16-row blocks that hold rows (k_contract_cc32 skips the rest)
-        for (const Work& w : p->comp_sched.works) issued += 64.0 * 16.0 * ((w.nrows + 15) / 16);
+        for (const OctWork& w : p->comp_sched.works) issued += 128.0 * 8.0 * w.tr;   // 128 pairs times 8 tr rows
         works = (double)p->comp_sched.works.size();
         nsplit = p->comp_sched.nsplit;
     }

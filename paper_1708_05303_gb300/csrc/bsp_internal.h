@@ -69,6 +69,23 @@ struct Work {
     int pad;
 };
 
+// FP32 contraction work item (k_contract_oct): 16 slots, each one shell b and
+// eight consecutive shells c (an octet), times rows that every slot lists for
+// itself, over fields staged once for all of them.
+constexpr int OCT_SLOTS = 16;
+constexpr int OCT_TRMAX = 7;                  // rows per thread; a slot has 8 of them
+constexpr int OCT_ROWS = 8 * OCT_TRMAX;
+constexpr int OCT_COLS = 8 * OCT_SLOTS;       // a CTA's partial sums: [OCT_ROWS][OCT_COLS] FP64
+struct OctWork {
+    int tr;             // rows per thread (1 .. OCT_TRMAX)
+    int nA;             // staged row fields
+    int nX;             // staged pair-factor shells
+    int stage0;         // their fields and shells: stage[stage0 .. + nA + nX)
+    int brow[OCT_SLOTS];   // staged index of the slot's b among the pair factors
+    int crow[OCT_SLOTS];   // ... and of its first c (the octet's eight are consecutive)
+    uint16_t arow[OCT_SLOTS][OCT_ROWS];   // staged index of each of the slot's rows
+};
+
 // One tensor-core work item: 128 pairs x N field rows (N = 8 nbox rounded up to 16).
 struct TcWork {
     int pair0, npairs;      // pairs [pair0, pair0 + npairs), npairs <= 128
@@ -129,11 +146,17 @@ struct ShotTerms {
 };
 
 // ---- launchers (bsp_contract.cu) ----
-template <typename R>
-cudaError_t launch_contract_cc(const R* rows, const R* px, const R* py, int sym, size_t fstride,
-                               const Work* works, int nwork, const int2* pair_fields,
-                               const int* row_fields, size_t npts, int nsplit, double* partial,
-                               cudaStream_t st);
+// FP64 contraction of the counts: rows x pair products of `pf`.
+cudaError_t launch_contract_f64(const double* rows, const double* pf, size_t fstride, const Work* works, int nwork,
+                                const int2* pair_fields, const int* row_fields, size_t npts, int nsplit,
+                                double* partial, cudaStream_t st);
+
+// FP32 contraction: rows: row fields (stage lists index them from `rows`);
+// the pair product of (b, c) is X_b Y_c + Y_b X_c with `sym`, else X_b X_c.
+// max_a, max_x: the most staged row fields and pair-factor shells of any work.
+cudaError_t launch_contract_oct(const float* rows, const float* px, const float* py, int sym, size_t fstride,
+                                const OctWork* works, int nwork, const int* stage, int max_a, int max_x, size_t npts,
+                                int nsplit, double* partial, cudaStream_t st);
 
 // Counts on the cubic group's orbit representatives: wrows[a][r] = w[r] *
 // fields[a][idx[r]], urows[a][r] = fields[a][idx[r]] (FP64, [nsh][nrep]).
