@@ -188,6 +188,10 @@ bsp_status bsp_modal_project(int n_keep, const double* gamma, int n_rhs, const d
  * bsp_covariance: mean (device FP64 [d]) and unbiased covariance (device
  *   FP64 [d][d]) of the m >= 2 rows of a device FP64 [m][d] matrix, two
  *   passes (mean, then centred products) in a fixed order.
+ * bsp_covariance_ws: the same with a device workspace of
+ *   bsp_covariance_workspace_size bytes (256-byte aligned; 0: none needed),
+ *   through which large matrices are multiplied on the tensor cores as exact
+ *   products of integer digits: no less accurate, and many times faster.
  */
 typedef struct bsp_batch bsp_batch;
 bsp_status bsp_batch_create(bsp_batch** out, int n_sizes, const int* sizes, double box, int n_shells,
@@ -202,6 +206,9 @@ bsp_status bsp_batch_bins(const bsp_batch* batch, int32_t* abc, double* counts);
 bsp_status bsp_batch_run(bsp_batch* batch, int n_mocks, const int* size_index, const void* const* delta_host,
                          void* ws, void* stream, double* rows);
 bsp_status bsp_covariance(int m, int d, const double* rows, double* mean, double* cov, void* stream);
+bsp_status bsp_covariance_workspace_size(int m, int d, size_t* bytes);
+bsp_status bsp_covariance_ws(int m, int d, const double* rows, double* mean, double* cov, void* ws,
+                             size_t ws_bytes, void* stream);
 
 /* Release the plan and its device tables (NULL is ignored). */
 void bsp_plan_destroy(bsp_plan* plan);

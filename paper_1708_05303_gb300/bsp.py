@@ -74,6 +74,8 @@ _SIGS = [
     ("bsp_batch_bins", ctypes.c_int, [_P, _P, _P]),
     ("bsp_batch_run", ctypes.c_int, [_P, ctypes.c_int, _P, _P, _P, _P, _P]),
     ("bsp_covariance", ctypes.c_int, [ctypes.c_int, ctypes.c_int, _P, _P, _P, _P]),
+    ("bsp_covariance_workspace_size", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_size_t)]),
+    ("bsp_covariance_ws", ctypes.c_int, [ctypes.c_int, ctypes.c_int, _P, _P, _P, _P, ctypes.c_size_t, _P]),
     ("bsp_plan_stats", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_double)]),
     ("bsp_set_profiling", ctypes.c_int, [_P, ctypes.c_int]),
     ("bsp_phase_times", ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int),
@@ -415,8 +417,13 @@ class Batch:
         m, d = rows.shape
         mean = torch.empty(d, dtype=torch.float64, device="cuda")
         cov = torch.empty((d, d), dtype=torch.float64, device="cuda")
-        _check(load().bsp_covariance(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _stream_handle(stream)),
-               "bsp_covariance")
+        nb = ctypes.c_size_t()
+        _check(load().bsp_covariance_workspace_size(int(m), int(d), ctypes.byref(nb)), "bsp_covariance")
+        ws = torch.empty(max(nb.value, 256), dtype=torch.uint8, device="cuda")
+        if stream is not None:
+            ws.record_stream(stream)   # released here, in use there
+        _check(load().bsp_covariance_ws(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _dptr(ws), int(nb.value),
+                                        _stream_handle(stream)), "bsp_covariance")
         return mean, cov
 
     def close(self):

@@ -1,6 +1,6 @@
-// bsp_batch.cu -- many mock realisations of uneven grid sizes, and the FP64
-// covariance of their multipoles (the use of mock catalogues for the
-// covariance, Sec. 1 and Sec. 3.1).
+// bsp_batch.cu -- many mock realisations of uneven grid sizes (the use of mock
+// catalogues for the covariance, Sec. 1 and Sec. 3.1; the covariance itself is
+// in bsp_cov.cu).
 //
 // One plan per grid size (the bins must coincide across sizes, so that the
 // multipole vectors of all mocks line up); all plans share one workspace,
@@ -24,54 +24,6 @@
 namespace {
 
 constexpr int MAX_SIZES = 8;
-
-__global__ void k_col_mean(const double* __restrict__ X, int m, int d, double* __restrict__ mean) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
-    double s = 0.0;
-    for (int i = 0; i < m; ++i) s += X[(size_t)i * d + j];
-    mean[j] = s / m;
-}
-
-// C[i][j] = sum_m (X[m][i] - mean[i]) (X[m][j] - mean[j]) / (m - 1), 32 x 32
-// tiles, upper triangle computed and mirrored; fixed summation order.
-__global__ void __launch_bounds__(256) k_cov(const double* __restrict__ X, const double* __restrict__ mean, int m,
-                                             int d, double* __restrict__ C) {
-    const int bi = blockIdx.y, bj = blockIdx.x;
-    if (bj < bi) return;
-    __shared__ double A[16][33], Bt[16][33];
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;   // 16 x 16 threads, 2 x 2 outputs each
-    double acc[2][2] = {{0, 0}, {0, 0}};
-    const int i0 = bi * 32, j0 = bj * 32;
-    for (int k0 = 0; k0 < m; k0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 32; e += 256) {
-            const int kk = e / 32, c = e % 32;
-            const int k = k0 + kk;
-            double a = 0.0, b = 0.0;
-            if (k < m && i0 + c < d) a = X[(size_t)k * d + i0 + c] - mean[i0 + c];
-            if (k < m && j0 + c < d) b = X[(size_t)k * d + j0 + c] - mean[j0 + c];
-            A[kk][c] = a;
-            Bt[kk][c] = b;
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < 16; ++kk)
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-#pragma unroll
-                for (int v = 0; v < 2; ++v) acc[u][v] = fma(A[kk][ty * 2 + u], Bt[kk][tx * 2 + v], acc[u][v]);
-        __syncthreads();
-    }
-    for (int u = 0; u < 2; ++u)
-        for (int v = 0; v < 2; ++v) {
-            const int i = i0 + ty * 2 + u, j = j0 + tx * 2 + v;
-            if (i < d && j < d) {
-                const double c = acc[u][v] / (m - 1);
-                C[(size_t)i * d + j] = c;
-                C[(size_t)j * d + i] = c;
-            }
-        }
-}
 
 }  // namespace
 
@@ -310,15 +262,6 @@ bsp_status bsp_batch_run(bsp_batch* bt, int n_mocks, const int* size_index, cons
             return BSP_ECUDA;
     }
     return BSP_OK;
-}
-
-bsp_status bsp_covariance(int m, int d, const double* rows, double* mean, double* cov, void* stream) {
-    if (m < 2 || d < 1 || !rows || !mean || !cov) return BSP_EINVAL;
-    cudaStream_t st = (cudaStream_t)stream;
-    k_col_mean<<<(d + 255) / 256, 256, 0, st>>>(rows, m, d, mean);
-    dim3 grid((d + 31) / 32, (d + 31) / 32);
-    k_cov<<<grid, 256, 0, st>>>(rows, mean, m, d, cov);
-    return cudaGetLastError() == cudaSuccess ? BSP_OK : BSP_ECUDA;
 }
 
 }  // extern "C"
