@@ -123,6 +123,96 @@ __device__ __forceinline__ void butterfly(cx<R>* v) {
     }
 }
 
+// FP32 arithmetic with every rounding written out.  Which product of a sum the
+// multiply-add takes is a choice of the compiler's that changes with the code
+// around it (by 1e-7 of a field); here it is fixed, so a transform has the same
+// bits whatever kernel it runs in.
+__device__ __forceinline__ cx<float> radd(cx<float> a, cx<float> b) { return {__fadd_rn(a.re, b.re), __fadd_rn(a.im, b.im)}; }
+__device__ __forceinline__ cx<float> rsub(cx<float> a, cx<float> b) { return {__fsub_rn(a.re, b.re), __fsub_rn(a.im, b.im)}; }
+__device__ __forceinline__ cx<float> rmul(cx<float> a, cx<float> b) {
+    return {__fmaf_rn(a.re, b.re, -__fmul_rn(a.im, b.im)), __fmaf_rn(a.im, b.re, __fmul_rn(a.re, b.im))};
+}
+// Inverse DFT of RADIX values in registers (as butterfly).
+template <int RADIX>
+__device__ __forceinline__ void dft(cx<float>* v) {
+    if constexpr (RADIX == 2) {
+        const cx<float> a = v[0], b = v[1];
+        v[0] = radd(a, b);
+        v[1] = rsub(a, b);
+    } else if constexpr (RADIX == 4) {
+        const cx<float> s02 = radd(v[0], v[2]), d02 = rsub(v[0], v[2]), s13 = radd(v[1], v[3]), d = rsub(v[1], v[3]);
+        const cx<float> d13 = {-d.im, d.re};
+        v[0] = radd(s02, s13);
+        v[2] = rsub(s02, s13);
+        v[1] = radd(d02, d13);
+        v[3] = rsub(d02, d13);
+    } else if constexpr (RADIX == 8) {
+        cx<float> e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        dft<4>(e);
+        dft<4>(o);
+        const float h = 0.70710678118654752440f;
+        const cx<float> u1 = {__fsub_rn(o[1].re, o[1].im), __fadd_rn(o[1].re, o[1].im)};
+        const cx<float> u3 = {-__fadd_rn(o[3].re, o[3].im), __fsub_rn(o[3].re, o[3].im)};
+        const cx<float> w2o = {-o[2].im, o[2].re};
+        v[0] = radd(e[0], o[0]);
+        v[4] = rsub(e[0], o[0]);
+        v[1] = {__fmaf_rn(u1.re, h, e[1].re), __fmaf_rn(u1.im, h, e[1].im)};
+        v[5] = {__fmaf_rn(-u1.re, h, e[1].re), __fmaf_rn(-u1.im, h, e[1].im)};
+        v[2] = radd(e[2], w2o);
+        v[6] = rsub(e[2], w2o);
+        v[3] = {__fmaf_rn(u3.re, h, e[3].re), __fmaf_rn(u3.im, h, e[3].im)};
+        v[7] = {__fmaf_rn(-u3.re, h, e[3].re), __fmaf_rn(-u3.im, h, e[3].im)};
+    } else if constexpr (RADIX == 16) {
+        const float c1 = 0.92387953251128675613f, s1 = 0.38268343236508977173f, h = 0.70710678118654752440f;
+        const cx<float> w[10] = {{1.f, 0.f}, {c1, s1}, {h, h}, {s1, c1}, {0.f, 1.f}, {-s1, c1}, {-h, h}, {-c1, s1}, {-1.f, 0.f}, {-c1, -s1}};
+        cx<float> a[4][4];
+#pragma unroll
+        for (int j2 = 0; j2 < 4; ++j2) {
+            cx<float> t[4] = {v[j2], v[j2 + 4], v[j2 + 8], v[j2 + 12]};
+            dft<4>(t);
+#pragma unroll
+            for (int k1 = 0; k1 < 4; ++k1) {
+                const int m = j2 * k1;
+                const cx<float> x = t[k1];
+                if (m == 0) a[j2][k1] = x;
+                else if (m == 4) a[j2][k1] = {-x.im, x.re};
+                else if (m == 2)
+                    a[j2][k1] = {__fmaf_rn(x.re, h, -__fmul_rn(x.im, h)), __fmaf_rn(x.re, h, __fmul_rn(x.im, h))};
+                else if (m == 6)
+                    a[j2][k1] = {__fmaf_rn(x.re, -h, -__fmul_rn(x.im, h)), __fmaf_rn(x.im, -h, __fmul_rn(x.re, h))};
+                else a[j2][k1] = rmul(x, w[m]);
+            }
+        }
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) {
+            cx<float> u[4] = {a[0][k1], a[1][k1], a[2][k1], a[3][k1]};
+            dft<4>(u);
+#pragma unroll
+            for (int k2 = 0; k2 < 4; ++k2) v[k1 + 4 * k2] = u[k2];
+        }
+    } else if constexpr (RADIX == 3) {
+        const float s3 = 0.86602540378443864676f;
+        const cx<float> t = radd(v[1], v[2]), d = rsub(v[1], v[2]);
+        const cx<float> m = {__fmaf_rn(-0.5f, t.re, v[0].re), __fmaf_rn(-0.5f, t.im, v[0].im)};
+        v[0] = radd(v[0], t);
+        v[1] = {__fmaf_rn(-d.im, s3, m.re), __fmaf_rn(d.re, s3, m.im)};
+        v[2] = {__fmaf_rn(d.im, s3, m.re), __fmaf_rn(-d.re, s3, m.im)};
+    } else if constexpr (RADIX == 5) {
+        const float c1 = 0.30901699437494742410f, c2 = -0.80901699437494742410f;
+        const float s1 = 0.95105651629515357212f, s2 = 0.58778525229247312917f;
+        const cx<float> t1 = radd(v[1], v[4]), d1 = rsub(v[1], v[4]), t2 = radd(v[2], v[3]), d2 = rsub(v[2], v[3]);
+        const cx<float> a1 = {__fmaf_rn(c2, t2.re, __fmaf_rn(c1, t1.re, v[0].re)), __fmaf_rn(c2, t2.im, __fmaf_rn(c1, t1.im, v[0].im))};
+        const cx<float> a2 = {__fmaf_rn(c1, t2.re, __fmaf_rn(c2, t1.re, v[0].re)), __fmaf_rn(c1, t2.im, __fmaf_rn(c2, t1.im, v[0].im))};
+        const cx<float> b1 = {-__fmaf_rn(s1, d1.im, __fmul_rn(s2, d2.im)), __fmaf_rn(s1, d1.re, __fmul_rn(s2, d2.re))};
+        const cx<float> b2 = {-__fmaf_rn(s2, d1.im, -__fmul_rn(s1, d2.im)), __fmaf_rn(s2, d1.re, -__fmul_rn(s1, d2.re))};
+        v[0] = radd(v[0], radd(t1, t2));
+        v[1] = radd(a1, b1);
+        v[4] = rsub(a1, b1);
+        v[2] = radd(a2, b2);
+        v[3] = rsub(a2, b2);
+    }
+}
+
 // Shared-memory layouts of P pencils of length M (one element = one complex):
 //   pencil-fast (passes 1, 2):  (p, i) -> i P + p + i/8
 //   index-fast  (pass 3):       (p, i) -> p PS + i + i/8,  PS = M + M/8 + 1
@@ -516,23 +606,6 @@ struct StageStockham {
         for (int i = 0; i < 4; ++i) v[i] = res[idx(p, m0 + i, M)];
     }
 };
-// Register pass 3 (M = 256): 16-element groups padded by 2 elements, lines
-// 288 elements apart, so the 4 elements of a 16-byte output chunk are two
-// aligned 16-byte loads and a quarter warp's loads fall on distinct banks.
-struct Stage3r {
-    static constexpr int PS = 288;
-    __device__ static int idx(int p, int m, int) { return p * PS + m + (m >> 4) * 2; }
-    template <typename R>
-    __device__ static void load4(const cx<R>* res, int p, int m0, int, cx<R> (&v)[4]) {
-        const float4* q = reinterpret_cast<const float4*>(res + idx(p, m0, 0));
-        const float4 a = q[0], b = q[1];
-        v[0] = {a.x, a.y};
-        v[1] = {a.z, a.w};
-        v[2] = {b.x, b.y};
-        v[3] = {b.z, b.w};
-    }
-};
-
 // Output of pass 3 for P consecutive y of one x: the real values of each
 // z-line, res[sidx<false, P>(p, m, M)] = F[2m] + i F[2m+1], scaled and
 // written as the field's FP32 row and/or 16-bit hi/lo planes.
@@ -707,67 +780,150 @@ __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restri
     pass3_store<R, P>(g, N, M, x, y0, res, fields[blockIdx.y], out, out_stride, hi, lo, f16, fmax2, f0max, lay);
 }
 
-// Pass 3 for n = 512 (M = 256 = 16 x 16) with the z-lines in registers:
-// 16 threads per line, P3R = 16 lines (consecutive y of one x) per CTA.
-// With k = k1 + 16 k2 and m = m1 + 16 m2,
-//   z_m = sum_k1 W16^{k1 m2} [ W256^{k1 m1} sum_k2 Z_{k1 + 16 k2} W16^{k2 m1} ],
-// W_L = e^{2 pi i / L}: thread k1 forms its 16 inputs Z_{k1 + 16 k2} straight
-// from T2 (the same Z_k as k_pass3), takes the inner 16-point DFT and the
-// twiddle in registers, the lines pass once through shared memory
-// (transposed), and thread m1 takes the outer 16-point DFT.  Two barriers
-// instead of one per Stockham stage, and every thread busy in both DFTs.
-constexpr int P3R = 16;
-constexpr int P3R_TS = 16 * 17;   // transpose rows per line: 16 rows of 16 + 1 pad
-constexpr int P3R_BUF = P3R * Stage3r::PS;   // staging buffer (the transpose fits in it)
-constexpr size_t p3r_smem_bytes() { return sizeof(cx<float>) * (512 + 256 + (size_t)P3R_BUF); }
-static_assert(P3R * P3R_TS <= P3R_BUF, "transpose fits in the output buffer");
 
-__global__ void __launch_bounds__(NTHR) k_pass3r(FftGeom g, const cx<float>* __restrict__ t2, size_t t2_stride,
-                                                 const cx<float>* __restrict__ twg,
-                                                 const FieldDesc* __restrict__ fields, float* __restrict__ out,
-                                                 size_t out_stride, uint32_t* __restrict__ hi,
-                                                 uint32_t* __restrict__ lo, int f16,
-                                                 const unsigned* __restrict__ fmax2,
-                                                 unsigned* __restrict__ f0max, FieldLayout lay) {
-    constexpr int N = 512, M = 256;
+// Pass 3 for the sizes known at compile time, FP32, with the z-lines in registers:
+// M = n/2 = R1 x R2, the two stages of the Stockham list (16 x 3, 16 x 4, 16 x 5,
+// 16 x 8, 16 x 16, 8 x 4).  P consecutive lines (of all n^2: T2 and the output are
+// both linear in the line) per CTA.  Thread (line, j < R2) forms its R1 inputs
+// Z_{j + R2 r} straight from T2 (the same Z_k as k_pass3) and takes the R1-point
+// DFT; the lines pass once through shared memory, and thread (line, j < R1)
+// takes the R2-point DFTs and stores from registers: 16 lanes hold 16
+// consecutive complex values, a whole 128-byte run of FP32 or 64 bytes of each
+// 16-bit plane row.  One barrier.  Eight lines a CTA through one shared-memory
+// stage after another, as before, kept a few dozen of 256 threads busy in the
+// radix-16 stage.  Fields and time before -> now: 288 FP32 fields of 256^3 14.2 ->
+// 4.9 ms (4.4 at the copy rate), 72 of 160^3 1.33 -> 0.27 ms, 150 operand sets of 256^3
+// 8.9 -> 4.4 ms, 96 of 512^3 (16 x 16 in registers before, staged for 16-byte stores)
+// 20.5 -> 18.8 ms.  Bound at 512^3: L1 wavefronts, 76 % busy (T2 rows of 1 040 bytes, the
+// 4-byte plane stores).
+template <int NN>
+struct P3V {
+    static constexpr int M = NN / 2;
+    static constexpr RadixList L = radix_list(M);
+    static constexpr int R1 = L.r[0], R2 = L.r[1];
+    static_assert(L.n == 2 && R1 * R2 == M, "two stages");
+    static constexpr int P = M >= 256 ? 16 : M >= 80 ? 32 : 64;   // divides n^2
+    static constexpr int T = P * R2;
+    // element i of a line at i + i / R1: stage 1 writes rows of R1 (odd row stride) and stage 2 reads columns
+    static constexpr int PS = M + R2;
+    __device__ static int idx(int p, int i) { return p * PS + i + i / R1; }
+    static constexpr size_t smem() { return sizeof(cx<float>) * ((size_t)P * PS + M); }
+};
+
+enum { P3_FIELD, P3_F16, P3_BF16 };   // FP32 fields, or the K-block-major operands with FP16 or BF16 planes
+
+template <int NN, int MODE>
+__global__ void __launch_bounds__(P3V<NN>::T) k_pass3v(FftGeom g, const cx<float>* __restrict__ t2, size_t t2_stride,
+                                                       const cx<float>* __restrict__ tw,
+                                                       const FieldDesc* __restrict__ fields, float* __restrict__ out,
+                                                       size_t out_stride, uint32_t* __restrict__ hi, int split,
+                                                       const unsigned* __restrict__ fmax2, FieldLayout lay) {
+    using V = P3V<NN>;
+    constexpr int M = V::M, R1 = V::R1, R2 = V::R2, P = V::P;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    cx<float>* tw = reinterpret_cast<cx<float>*>(smem_raw);
-    cx<float>* tw2 = tw + N;     // [m1][t] = W256^{t m1}: conflict-free reads across t
-    cx<float>* buf = tw2 + 256;
-    const int x = blockIdx.x / (N / P3R), y0 = (blockIdx.x % (N / P3R)) * P3R;
-    const int p = threadIdx.x >> 4, t = threadIdx.x & 15;
-    for (int i = threadIdx.x; i < N; i += NTHR) tw[i] = twg[i];
-    tw2[threadIdx.x] = twg[(2 * (threadIdx.x & 15) * (threadIdx.x >> 4)) & (N - 1)];
-    __syncthreads();
-    const int nKz = g.nKz;
-    const int nk = field_ext(fields[blockIdx.y], g) + 1;   // f_z read: 0 .. nk - 1
-    const cx<float>* h = t2 + (size_t)blockIdx.y * t2_stride + ((size_t)x * N + y0 + p) * nKz;
-    cx<float> v[16];
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    cx<float>* tw2 = buf + P * V::PS;   // [r][j] = W_M^{r j}: consecutive across the lanes (gathered from global
+                                        // memory at each use, they took most of the L1 wavefronts)
+    const FieldDesc fd = fields[blockIdx.y];
+    const int nKz = g.nKz, nk = field_ext(fd, g) + 1;   // f_z read: 0 .. nk - 1
+    const size_t line0 = (size_t)blockIdx.x * P;
+    for (int i = threadIdx.x; i < M; i += V::T) tw2[i] = tw[2 * (i / R1) * (i % R1)];
+    {
+        const int j = threadIdx.x % R2, p = threadIdx.x / R2;
+        const cx<float>* h = t2 + (size_t)blockIdx.y * t2_stride + (line0 + p) * nKz;
+        cx<float> v[R1];
 #pragma unroll
-    for (int k2 = 0; k2 < 16; ++k2) {
-        const int k = t + 16 * k2;
-        cx<float> a = {0.f, 0.f}, b = {0.f, 0.f};
-        if (k < nk) a = h[k];
-        if (M - k < nk) b = h[M - k];
-        if (k == 0) { a.im = 0.f; b.im = 0.f; }   // H_0 and H_M: real parts only
-        const cx<float> bc = {b.re, -b.im};
-        const cx<float> s = cadd(a, bc), d = csub(a, bc);
-        v[k2] = cadd(s, cmuli(cmul(d, tw[k])));
+        for (int r = 0; r < R1; ++r) {
+            const int k = j + R2 * r;
+            cx<float> a = {0.f, 0.f}, b = {0.f, 0.f};
+            if (k < nk) a = h[k];
+            if (M - k < nk) b = h[M - k];
+            if (k == 0) { a.im = 0.f; b.im = 0.f; }   // H_0 and H_M: real parts only
+            const cx<float> bc = {b.re, -b.im};
+            const cx<float> s = radd(a, bc), d = rsub(a, bc), dw = rmul(d, tw[k]);
+            v[r] = radd(s, cx<float>{-dw.im, dw.re});
+        }
+        dft<R1>(v);
+#pragma unroll
+        for (int r = 0; r < R1; ++r) buf[V::idx(p, j * R1 + r)] = v[r];
     }
-    butterfly<float, 16>(v);   // v[m1] = sum_k2 Z_{t + 16 k2} W16^{k2 m1}
-    cx<float>* tr = buf + p * P3R_TS;
-#pragma unroll
-    for (int m1 = 0; m1 < 16; ++m1) tr[m1 * 17 + t] = m1 == 0 ? v[0] : cmul(v[m1], tw2[m1 * 16 + t]);   // W256^{t m1}
     __syncthreads();
+    // the power-of-two scales of the tensor-core operands (see pass3_store)
+    float sc = 1.f, s7 = 1.f;
+    if (MODE != P3_FIELD) {
+        const float bound = 2.f * (float)nKz * __uint_as_float(fmax2[fd.out16]);
+        sc = pow2_scale(bound);
+        s7 = pow2_scale(bound, 7);
+    }
+#pragma unroll 1
+    for (int e = threadIdx.x; e < P * R1; e += V::T) {
+        const int j = e % R1, p = e / R1;
+        cx<float> v[R2];
 #pragma unroll
-    for (int k1 = 0; k1 < 16; ++k1) v[k1] = tr[t * 17 + k1];
-    butterfly<float, 16>(v);   // v[m2] = z_{t + 16 m2}
-    __syncthreads();           // every line's transpose is read before the output layout reuses it
+        for (int r = 0; r < R2; ++r) {
+            const cx<float> x = buf[V::idx(p, j + R1 * r)];
+            v[r] = r == 0 ? x : rmul(x, tw2[r * R1 + j]);
+        }
+        dft<R2>(v);
+        const size_t pos0 = (line0 + p) * M + j;   // complex values: pairs of consecutive z
+        if (MODE == P3_FIELD) {
+            cx<float>* d = reinterpret_cast<cx<float>*>(out + (size_t)fd.out32 * out_stride) + pos0;
 #pragma unroll
-    for (int m2 = 0; m2 < 16; ++m2) buf[Stage3r::idx(p, t + 16 * m2, M)] = v[m2];
-    __syncthreads();
-    pass3_store<float, P3R, Stage3r>(g, N, M, x, y0, buf, fields[blockIdx.y], out, out_stride, hi, lo, f16, fmax2,
-                                     f0max, lay);
+            for (int r = 0; r < R2; ++r) d[R1 * r] = v[r];
+            continue;
+        }
+        // Value r is pair w = pos % 32 of K-block pos / 32 (points 2 w, 2 w + 1).  pos0 - j is a
+        // multiple of R1; where a line is whole K-blocks (M = 32, 64, ...), w depends on r
+        // through r R1 % 32 only.
+        const size_t kb0 = pos0 >> 5;
+        const int w0 = (int)(pos0 & 31);
+        auto at = [&](int r, size_t& kb, int& w) {
+            if (M % 32 == 0) {
+                kb = kb0 + (R1 * r) / 32;
+                w = j + (R1 * r) % 32;
+            } else {
+                kb = kb0 + ((w0 + R1 * r) >> 5);
+                w = (w0 + R1 * r) & 31;
+            }
+        };
+        if (fd.out32 >= 0) {   // FP32 row: 16-byte chunk J of 256 bytes, swizzled in halves
+            const int r32 = fd.out32 & 7;
+            cx<float>* d = reinterpret_cast<cx<float>*>(out) + (size_t)fd.out32 * 32;
+#pragma unroll
+            for (int r = 0; r < R2; ++r) {
+                size_t kb;
+                int w;
+                at(r, kb, w);
+                d[kb * (size_t)(lay.rows32 * 32) + (w ^ (2 * r32))] = cx<float>{v[r].re * s7, v[r].im * s7};
+            }
+        }
+        uint32_t* q = hi + (size_t)(fd.out16 >> 3) * 512 + (size_t)(fd.out16 & 7) * 32;
+        const int r16 = fd.out16 & 7;
+#pragma unroll
+        for (int r = 0; r < R2; ++r) {   // plane rows: 16-byte chunks swizzled; the lo row 1024 bytes further
+            size_t kb;
+            int w;
+            at(r, kb, w);
+            uint32_t* d = q + kb * (size_t)(lay.groups16 * 512) + (w ^ (4 * r16));
+            const float x0 = v[r].re * sc, x1 = v[r].im * sc;
+            uint32_t hw, lw;
+            float h0, h1;
+            if (MODE == P3_F16) {
+                asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
+                unsigned short a = (unsigned short)(hw & 0xFFFFu), b = (unsigned short)(hw >> 16);
+                asm("cvt.f32.f16 %0, %1;" : "=f"(h0) : "h"(a));
+                asm("cvt.f32.f16 %0, %1;" : "=f"(h1) : "h"(b));
+                asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
+            } else {
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
+                h0 = __uint_as_float(hw << 16);
+                h1 = __uint_as_float(hw & 0xFFFF0000u);
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
+            }
+            d[0] = hw;
+            if (split) d[256] = lw;
+        }
+    }
 }
 
 template <typename R>
@@ -806,11 +962,13 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
             return e;
         set12 = sm12;
     }
-    if (sm3 > set3) {
-        if ((e = cudaFuncSetAttribute(k_pass3<R, C::P3, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm3)) != cudaSuccess)
-            return e;
-        set3 = sm3;
+    if constexpr (NN == 0 || !std::is_same<R, float>::value) {
+        if (sm3 > set3) {
+            if ((e = cudaFuncSetAttribute(k_pass3<R, C::P3, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)sm3)) != cudaSuccess)
+                return e;
+            set3 = sm3;
+        }
     }
     const int nkzb = (g.nKz + C::P - 1) / C::P;
     dim3 g1(g.nK * nkzb, nfields), g2(N * nkzb, nfields), g3(N * ((N + C::P3 - 1) / C::P3), nfields);
@@ -840,17 +998,13 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
     } else {
         k_pass2<R, C::P, NN><<<g2, NTHR, sm12, st>>>(g, t1, t1_stride, tw, t2, t2_stride, d_fields, fmax2);
     }
-    if constexpr (NN == 512 && std::is_same<R, float>::value) {
-        static bool set3r = false;
-        if (!set3r) {
-            if ((e = cudaFuncSetAttribute(k_pass3r, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)p3r_smem_bytes())) != cudaSuccess)
-                return e;
-            set3r = true;
-        }
-        k_pass3r<<<dim3(N * (N / P3R), nfields), NTHR, p3r_smem_bytes(), st>>>(g, t2, t2_stride, tw, d_fields, out,
-                                                                               out_stride, hi, lo, f16, fmax2,
-                                                                               f0max, lay);
+    if constexpr (NN > 0 && std::is_same<R, float>::value) {
+        using V = P3V<NN>;
+        const dim3 gv((unsigned)((size_t)N * N / V::P), nfields);
+        const bool kbm = lay.groups16 > 0;
+        auto kern = !kbm ? k_pass3v<NN, P3_FIELD> : f16 ? k_pass3v<NN, P3_F16> : k_pass3v<NN, P3_BF16>;
+        kern<<<gv, V::T, V::smem(), st>>>(g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo != nullptr, fmax2,
+                                          lay);
     } else {
         k_pass3<R, C::P3, NN><<<g3, NTHR, sm3, st>>>(g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo, f16,
                                                      fmax2, f0max, lay);
