@@ -25,7 +25,7 @@
 //               and every FLUSH_KB K-blocks add that sum, unscaled,
 //               to the CTA's FP64 slot in global memory (fire-and-forget
 //               reductions).
-// Two accumulator buffers and two A buffers in tensor memory keep TMA, the
+// Two accumulator buffers and three A buffers in tensor memory keep TMA, the
 // CUDA-core prologue, the MMAs and the epilogue overlapped.  Every mbarrier
 // wait is bounded; on timeout the CTA records an error code, stops, waits
 // (bounded) for its own copies in flight and releases its tensor memory.
@@ -43,29 +43,28 @@ constexpr int TC_SLOT = 128 * 128;   // FP64 values per CTA slot of the partial 
 constexpr int TC_KB = 64;        // x-points per K-block (128 bytes of 16-bit values)
 constexpr int NT = 4;            // TMA ring stages (F0 rows + field planes)
 constexpr int TC_MAXSH = 64;     // F0 rows per tile
-#ifndef TC_PRO_WARPS
-#define TC_PRO_WARPS 8
-#endif
-// warps: 0 copies, 1 MMA, 4 .. 4 + N_PRO - 1 pair products (N_PRO / 4 per TMEM
-// lane quadrant, each a 64 / (N_PRO / 4)-point part of every K-block), then 8 drain warps
-constexpr int N_PRO = TC_PRO_WARPS, PRO_PTS = 64 / (N_PRO / 4), PRO_CH = PRO_PTS / 4;
+// warps: 0 copies, 1 MMA, 4 .. 11 pair products (two per TMEM lane quadrant, each 32
+// points of every K-block), then 8 drain warps
+constexpr int N_PRO = 8, PRO_PTS = 64 / (N_PRO / 4), PRO_CH = PRO_PTS / 4;
 // 8 drain warps: warp 12 + 4 h + q reads columns [48 h, 48 h + 48) of lane
 // quadrant q and keeps their running sum in registers
 constexpr int W_TMA = 0, W_MMA = 1, W_PRO0 = 4, W_EPI0 = W_PRO0 + N_PRO, N_EPI = 8, EPI_COLS = 48;
 constexpr int TC_THREADS = 32 * (W_EPI0 + N_EPI);
-static_assert(N_PRO == 8 || N_PRO == 16, "pair-product warps: 8 or 16");
 // tensor memory columns: the P_hi F_hi accumulators D0 [0,96) and D1 [96,192),
 // drained every chunk; the correction accumulator E = P_hi F_lo + P_lo F_hi
-// [192,288), drained every CORR_KB K-blocks; two A buffers [288,352) and
-// [352,416), hi in the first 32 columns, lo in the next 32.  The running FP32
-// sum of the drained accumulators lives in the drain warps' registers.
+// [192,288), drained every CORR_KB K-blocks; three A buffers [288,480), hi in the
+// first 32 columns of each, lo in the next 32.  The running FP32 sum of the drained
+// accumulators lives in the drain warps' registers.
 // E's terms are ~2^-11 of D's: kept apart, the tensor core's truncating FP32
 // accumulation does not lose half an ulp of D on each correction product.
-// With the MMAs issued by an elected lane of the whole warp (below), the 12
-// MMAs of a split K-block issue in ~320 cycles and complete ~500 later, so a
-// third A buffer no longer shortens the chain products -> MMAs -> products.
 constexpr uint32_t TMEM_COLS = 512, COL_ACC = 96, COL_CORR = 192, COL_A = 288;
-constexpr int NA = 2;            // A buffers (pair products) in tensor memory
+// A buffers (pair products) in tensor memory.  With two, and the products begun only
+// when a buffer was free, a K-block's period was half the loop MMAs (N-dependent,
+// ~1 150 cycles at N = 96) -> products -> MMAs: 1 370 (N = 32) to 1 880 cycles (N = 96).
+// With three, and only the stores waiting for the buffer, it is 1 220 to 1 320,
+// nearly flat in N: the issue slots (~73 % used) and the drain bound it now.
+// Sixteen product warps (setmaxnreg shares) were slower (1 330 to 1 450).
+constexpr int NA = 3;
 constexpr int CORR_KB = 64;      // K-blocks per drain of E (a multiple of the chunk)
 constexpr int FLUSH_KB = 128;    // K-blocks between FP64 flushes of the running sum
 
@@ -110,11 +109,6 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
         "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
         : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-                 "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-                 : "memory");
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -180,6 +174,9 @@ __device__ __forceinline__ uint64_t pack64(float x0, float x1) {
     uint64_t d;
     asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x0), "f"(x1));
     return d;
+}
+__device__ __forceinline__ void lds_2x64(uint32_t addr, uint64_t& a, uint64_t& b) {
+    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr));
 }
 __device__ __forceinline__ void unpack64(uint64_t v, float& x0, float& x1) {
     asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(v));
@@ -292,39 +289,42 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const uint32_t tmem = S.tmem_base;
 
     if (warp == W_TMA) {
-        if (lane == 0) {
-            const int npc = S.npc;
-            const uint32_t f0_bytes = (uint32_t)w.nshell * 256;
-            const uint32_t bytes = f0_bytes + (uint32_t)w.nbox * 2048;
-            const uint8_t* f0src = reinterpret_cast<const uint8_t*>(gf0) + (size_t)(f0_row0 + w.shell_lo) * 256;
-            const uint8_t* psrc = reinterpret_cast<const uint8_t*>(gplanes);
-            int issued = 0;
-            for (int k = 0; k < nkb && !S.abort; ++k) {
-                const int s = k % NT, u = k / NT;
-                if (u > 0 && !mbar_wait(&S.kb_done[s], (u - 1) & 1, wlim)) {
-                    set_abort(S, err, 1);
-                    break;
-                }
-                const int sup = k / unit.len, kin = k % unit.len;
-                const long long kb = (long long)sup * lsup + unit.start + kin;
-                if (kb < nkb_real) {
-                    mbar_expect_tx(&S.tma_full[s], bytes);
-                    bulk_load(S.f0[s], f0src + (size_t)kb * f0_rows * 256, f0_bytes, &S.tma_full[s]);
-                    for (int j = 0; j < npc; ++j) {
-                        const int4 c = S.pc[j];
-                        bulk_load(&S.b[s][c.y * 2048], psrc + ((size_t)kb * groups + c.x) * 2048,
-                                  (uint32_t)c.z * 2048, &S.tma_full[s]);
-                    }
-                } else {
-                    mbar_expect_tx(&S.tma_full[s], 0);   // past the grid: nothing to load
-                }
-                issued = k + 1;
+        // lane 0 copies the F0 rows, lanes 1 .. npc one run of plane groups each, all in
+        // one instruction per K-block
+        const bool mine = lane <= S.npc;
+        const uint32_t f0_bytes = (uint32_t)w.nshell * 256;
+        const uint32_t bytes = f0_bytes + (uint32_t)w.nbox * 2048;
+        const int4 c = mine && lane ? S.pc[lane - 1] : make_int4(0, 0, 0, 0);
+        const uint8_t* src = lane == 0 ? reinterpret_cast<const uint8_t*>(gf0) + (size_t)(f0_row0 + w.shell_lo) * 256
+                                       : reinterpret_cast<const uint8_t*>(gplanes) + (size_t)c.x * 2048;
+        const size_t step = lane == 0 ? (size_t)f0_rows * 256 : (size_t)groups * 2048;
+        uint8_t* dst = lane == 0 ? S.f0[0] : &S.b[0][c.y * 2048];
+        const uint32_t dstep = lane == 0 ? (uint32_t)sizeof(S.f0[0]) : (uint32_t)sizeof(S.b[0]);
+        const uint32_t sz = lane == 0 ? f0_bytes : (uint32_t)c.z * 2048;
+        int issued = 0;
+        long long kb = unit.start;
+        for (int k = 0, kin = 0; k < nkb; ++k) {
+            const int s = k % NT, u = k / NT;
+            if (u > 0 && !warp_wait<1>(smem_u32(&S.kb_done[s]), (u - 1) & 1, wlim, &S.abort)) {
+                if (lane == 0) set_abort(S, err, 1);
+                break;
             }
-            // copies in flight must land before the CTA can exit: the last use of each
-            // stage (always the long limit, whatever the pipeline waits use)
+            const bool real = kb < nkb_real;   // past the grid: nothing to load
+            if (lane == 0) mbar_expect_tx(&S.tma_full[s], real ? bytes : 0u);
+            __syncwarp();
+            if (real && mine) bulk_load(dst + (size_t)s * dstep, src + (size_t)kb * step, sz, &S.tma_full[s]);
+            issued = k + 1;
+            ++kb;
+            if (++kin == unit.len) {
+                kin = 0;
+                kb += lsup - unit.len;
+            }
+        }
+        // copies in flight must land before the CTA can exit: the last use of each
+        // stage (always the long limit, whatever the pipeline waits use)
+        if (lane == 0)
             for (int k = max(0, issued - NT); k < issued; ++k)
                 if (!mbar_wait(&S.tma_full[k % NT], (k / NT) & 1)) atomicOr(err, 16);
-        }
     } else if (warp == W_MMA) {
         // the whole warp walks the K-blocks (the loop state stays warp-uniform);
         // one elected lane issues the MMAs and commits
@@ -336,25 +336,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const uint32_t dlo0 = (uint32_t)sw128_desc(smem_u32(S.b[0]), 2048);
         constexpr uint32_t STAGE16 = (uint32_t)(sizeof(S.b[0]) >> 4);
         int done = 0, kc = 0, c = 0;   // kc = k % CHUNK, c = k / CHUNK
-        bool ok = true;
-        for (int k = 0; k < nkb; ++k) {
-            const int s = k % NT, u = k / NT, sa = k % NA;
+        int ce = 0, ep = 0;            // ce = c % CC, ep = c / CC: chunk of the drain period of E, and the period
+        for (int k = 0, sa = 0, ua = 0; k < nkb; ++k) {   // sa = k % NA, ua = k / NA
+            const int s = k % NT, u = k / NT;
             const int j = c & 1;
-            const bool efirst = kc == 0 && c % CC == 0;   // first K-block of a drain period of E
-            if (kc == 0 && c >= 2 && !__all_sync(0xffffffffu, mbar_wait(&S.acc_empty[j], ((c >> 1) - 1) & 1, wlim))) {
-                ok = false;
-                break;
+            const bool efirst = kc == 0 && ce == 0;   // first K-block of a drain period of E
+            // the K-block's copies and pair products, and where it starts a chunk (a drain
+            // period of E) the accumulator read out: one barrier per lane
+            uint32_t bar = smem_u32(&S.tma_full[s]), par = (uint32_t)(u & 1);
+            if ((lane & 3) == 1) {
+                bar = smem_u32(&S.a_full[sa]);
+                par = (uint32_t)(ua & 1);
+            } else if ((lane & 3) == 2 && kc == 0 && c >= 2) {
+                bar = smem_u32(&S.acc_empty[j]);
+                par = (uint32_t)(((c >> 1) - 1) & 1);
+            } else if ((lane & 3) == 3 && nprod == 3 && efirst && c > 0) {
+                bar = smem_u32(&S.corr_empty);
+                par = (uint32_t)((ep - 1) & 1);
             }
-            if (nprod == 3 && efirst && c > 0 &&
-                !__all_sync(0xffffffffu, mbar_wait(&S.corr_empty, ((c / CC) - 1) & 1, wlim))) {
-                ok = false;
-                break;
-            }
-            if (!__all_sync(0xffffffffu, mbar_wait(&S.tma_full[s], u & 1, wlim) && mbar_wait(&S.a_full[sa], (k / NA) & 1, wlim))) {
+            if (!warp_wait<64>(bar, par, wlim, &S.abort)) {
                 if (lane == 0) set_abort(S, err, 4);
                 break;
             }
-            if (__shfl_sync(0xffffffffu, S.abort, 0)) break;
             tc_fence_after();
             if (elect_one()) {
                 const uint32_t d = tmem + (uint32_t)j * COL_ACC, de = tmem + COL_CORR;
@@ -376,10 +379,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             if (++kc == CHUNK || k == nkb - 1) {
                 kc = 0;
                 ++c;
+                if (++ce == CC) {
+                    ce = 0;
+                    ++ep;
+                }
+            }
+            if (++sa == NA) {
+                sa = 0;
+                ++ua;
             }
             done = k + 1;
         }
-        if (!ok && lane == 0) set_abort(S, err, 2);
         // the last MMAs must finish before tensor memory is released (long limit)
         if (done > 0 && !__all_sync(0xffffffffu, mbar_wait(&S.kb_done[(done - 1) % NT], ((done - 1) / NT) & 1)) && lane == 0)
             atomicOr(err, 32);
@@ -391,57 +401,67 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const int2 bc = S.pf[i];
         const bool pair = bc.x >= 0;
         const int rb = pair ? bc.x : 0, rc = pair ? bc.y : 0;
-        // F0 row r (relative to the tile's first shell, absolute K-block row g = f0_row0 +
-        // shell_lo + r): 16-byte chunk j of half h at r*256 + 128 h + ((j ^ (g & 7)) << 4)
+        // F0 row r (relative to the tile's first shell, absolute K-block row g = f0_row0 + shell_lo + r):
         const int g0 = f0_row0 + w.shell_lo;
-        const int ob = rb * 256 + 128 * h, sb = (g0 + rb) & 7, oc = rc * 256 + 128 * h, sc = (g0 + rc) & 7;
+        // chunk j at row base + ((j ^ (g & 7)) << 4): the bases hold (g & 7) << 4, and a K-block's
+        // chunk addresses differ from them in those bits only
+        const uint32_t xb = smem_u32(S.f0[0]) + (uint32_t)(rb * 256 + 128 * h + (((g0 + rb) & 7) << 4));
+        const uint32_t xc = smem_u32(S.f0[0]) + (uint32_t)(rc * 256 + 128 * h + (((g0 + rc) & 7) << 4));
         const uint32_t lanebase = ((uint32_t)(32 * q) << 16) + (uint32_t)(t * PRO_PTS / 2);
-        for (int k = 0; k < nkb && !S.abort; ++k) {
-            const int s = k % NT, u = k / NT, sa = k % NA;
-            if (!mbar_wait(&S.tma_full[s], u & 1, wlim) ||
-                (k >= NA && !mbar_wait(&S.kb_done[(k - NA) % NT], ((k - NA) / NT) & 1, wlim))) {
-                set_abort(S, err, 8);
+        long long kb = unit.start;
+        for (int k = 0, kin = 0, sa = 0; k < nkb; ++k) {   // sa = k % NA
+            const int s = k % NT, u = k / NT;
+            if (!warp_wait<1>(smem_u32(&S.tma_full[s]), (uint32_t)(u & 1), wlim, &S.abort)) {
+                if (lane == 0) set_abort(S, err, 8);
+                break;
+            }
+            const bool real = kb < nkb_real;   // past the grid: products of zero (rows without a pair hold anything)
+            ++kb;
+            if (++kin == unit.len) {
+                kin = 0;
+                kb += lsup - unit.len;
+            }
+            const uint32_t sb = xb + (uint32_t)s * (uint32_t)sizeof(S.f0[0]), sc = xc + (uint32_t)s * (uint32_t)sizeof(S.f0[0]);
+            uint32_t vh[2 * PRO_CH], vl[2 * PRO_CH];
+            if (real) {
+#pragma unroll
+                for (int jj = 0; jj < PRO_CH; ++jj) {
+                    const uint32_t jx = (uint32_t)(j0 + jj) << 4;
+                    uint64_t b01, b23, c01, c23;
+                    lds_2x64(sb ^ jx, b01, b23);
+                    lds_2x64(sc ^ jx, c01, c23);
+                    const uint64_t p01 = fmul2(b01, c01), p23 = fmul2(b23, c23);
+                    float p0, p1, p2, p3, h0, h1, h2, h3;
+                    unpack64(p01, p0, p1);
+                    unpack64(p23, p2, p3);
+                    vh[2 * jj] = pack2<F16>(p0, p1);
+                    vh[2 * jj + 1] = pack2<F16>(p2, p3);
+                    unpack2<F16>(vh[2 * jj], h0, h1);
+                    unpack2<F16>(vh[2 * jj + 1], h2, h3);
+                    float r0, r1, r2, r3;
+                    unpack64(fsub2(p01, pack64(h0, h1)), r0, r1);
+                    unpack64(fsub2(p23, pack64(h2, h3)), r2, r3);
+                    vl[2 * jj] = pack2<F16>(r0, r1);
+                    vl[2 * jj + 1] = pack2<F16>(r2, r3);
+                }
+            } else {
+#pragma unroll
+                for (int jj = 0; jj < 2 * PRO_CH; ++jj) vh[jj] = vl[jj] = 0u;
+            }
+            // only the stores need the A buffer: the MMAs that read it before may still run meanwhile
+            if (k >= NA && !warp_wait<1>(smem_u32(&S.kb_done[(k - NA) % NT]), (uint32_t)(((k - NA) / NT) & 1), wlim, &S.abort)) {
+                if (lane == 0) set_abort(S, err, 8);
                 break;
             }
             tc_fence_after();
-            const bool live = pair && (long long)(k / unit.len) * lsup + unit.start + k % unit.len < nkb_real;
-            const uint8_t* f0 = S.f0[s];
-            uint32_t vh[2 * PRO_CH], vl[2 * PRO_CH];
-#pragma unroll
-            for (int jj = 0; jj < PRO_CH; ++jj) {
-                const int j = j0 + jj;
-                uint64_t p01 = 0, p23 = 0;
-                if (live) {
-                    const float4 fb = *reinterpret_cast<const float4*>(f0 + ob + ((j ^ sb) << 4));
-                    const float4 fc = *reinterpret_cast<const float4*>(f0 + oc + ((j ^ sc) << 4));
-                    p01 = fmul2(pack64(fb.x, fb.y), pack64(fc.x, fc.y));
-                    p23 = fmul2(pack64(fb.z, fb.w), pack64(fc.z, fc.w));
-                }
-                float p0, p1, p2, p3, h0, h1, h2, h3;
-                unpack64(p01, p0, p1);
-                unpack64(p23, p2, p3);
-                vh[2 * jj] = pack2<F16>(p0, p1);
-                vh[2 * jj + 1] = pack2<F16>(p2, p3);
-                unpack2<F16>(vh[2 * jj], h0, h1);
-                unpack2<F16>(vh[2 * jj + 1], h2, h3);
-                float r0, r1, r2, r3;
-                unpack64(fsub2(p01, pack64(h0, h1)), r0, r1);
-                unpack64(fsub2(p23, pack64(h2, h3)), r2, r3);
-                vl[2 * jj] = pack2<F16>(r0, r1);
-                vl[2 * jj + 1] = pack2<F16>(r2, r3);
-            }
             const uint32_t ta = tmem + lanebase + COL_A + (uint32_t)sa * 64;
-            if constexpr (PRO_CH == 4) {
-                tmem_st8(ta, *reinterpret_cast<const uint32_t(*)[8]>(vh));
-                if (nprod == 3) tmem_st8(ta + 32, *reinterpret_cast<const uint32_t(*)[8]>(vl));
-            } else {
-                tmem_st16(ta, *reinterpret_cast<const uint32_t(*)[16]>(vh));
-                if (nprod == 3) tmem_st16(ta + 32, *reinterpret_cast<const uint32_t(*)[16]>(vl));
-            }
+            tmem_st16(ta, vh);
+            if (nprod == 3) tmem_st16(ta + 32, vl);
             tmem_st_wait();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&S.a_full[sa]);
+            sa = sa == NA - 1 ? 0 : sa + 1;
         }
     } else if (warp >= W_EPI0) {
         const int q = warp & 3, hc = (warp - W_EPI0) >> 2;
@@ -455,16 +475,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         float sum[EPI_COLS];
 #pragma unroll
         for (int t = 0; t < EPI_COLS; ++t) sum[t] = 0.f;
-        for (int c = 0; c < nch && !S.abort; ++c) {
-            const int j = c & 1, g = c % FL;
+        for (int c = 0, g = 0, ce = 0; c < nch; ++c) {
+            const int j = c & 1;   // g = c % FL, ce = c % CC
             const bool flush = g == FL - 1 || c == nch - 1;
-            if (!mbar_wait(&S.acc_full[j], (c >> 1) & 1, wlim)) {
-                set_abort(S, err, 64);
+            g = g == FL - 1 ? 0 : g + 1;
+            if (!warp_wait<1>(smem_u32(&S.acc_full[j]), (uint32_t)((c >> 1) & 1), wlim, &S.abort)) {
+                if (lane == 0) set_abort(S, err, 64);
                 break;
             }
             tc_fence_after();
             // every CC chunks, and at the end, E joins the running sum first
-            if (nprod == 3 && ((c + 1) % CC == 0 || c == nch - 1)) {
+            const bool edrain = ce == CC - 1 || c == nch - 1;
+            ce = ce == CC - 1 ? 0 : ce + 1;
+            if (nprod == 3 && edrain) {
 #pragma unroll
                 for (int cg = 0; cg < EPI_COLS / 16; ++cg) {
                     const uint32_t col = c0 + 16u * cg;
