@@ -599,8 +599,8 @@ struct bsp_plan {
 namespace {
 
 void t12_sizes(const FftGeom& g, size_t elem, size_t* t1, size_t* t2) {
-    *t1 = round256((size_t)g.nK * g.n * g.nKz * 2 * elem);
-    *t2 = round256((size_t)g.n * g.n * g.nKz * 2 * elem);
+    *t1 = round256((size_t)g.nK * g.n * g.ldz * 2 * elem);
+    *t2 = round256((size_t)g.n * g.n * g.ldz * 2 * elem);
 }
 
 // Offsets inside the workspace (the same for counts and compute; the two
@@ -764,6 +764,7 @@ bsp_status bsp_plan_create(bsp_plan** out, int n, double box, int n_shells, cons
     } else {
         g.K = K; g.nK = 2 * K + 1; g.pruned = 1; g.nKz = K + 1;
     }
+    g.ldz = (g.nKz + 7) & ~7;
     g.n2max = 3 * (n / 2) * (n / 2);
     if (!radix_plan(n, g.rad, &g.nrad) || !radix_plan(n / 2, g.rad_h, &g.nrad_h)) {
         delete p;
@@ -950,6 +951,7 @@ bsp_status bsp_plan_create_modal(bsp_plan** out, int n, double box, int n_funcs,
     } else {
         g.K = K; g.nK = 2 * K + 1; g.pruned = 1; g.nKz = K + 1;
     }
+    g.ldz = (g.nKz + 7) & ~7;
     g.n2max = n2max;
     if (!radix_plan(n, g.rad, &g.nrad) || !radix_plan(n / 2, g.rad_h, &g.nrad_h)) {
         delete p;
@@ -1131,8 +1133,7 @@ bsp_status bsp_counts(bsp_plan* p, void* ws, void* stream) {
     for (int f0 = 0; f0 < p->nsh; f0 += p->fb64) {
         int nf = std::min(p->fb64, p->nsh - f0);
         cudaError_t e = launch_fft_fields<double>(p->geom, nullptr, p->d_shell_of, nullptr, p->d_fd_unit + f0, nf,
-                                                  p->d_tw64, t1, t2, f64, p->npts(), nullptr, nullptr, 0, nullptr,
-                                                  nullptr, st);
+                                                  p->d_tw64, t1, t2, f64, p->npts(), nullptr, nullptr, 0, nullptr, st);
         if (e != cudaSuccess) return cuda_fail(e, "fft (counts)");
     }
     // gather the unit fields on the representatives of the cubic group's
@@ -1250,7 +1251,7 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
             int nb = std::min(p->fb32, nf - f0i);
             cudaError_t e = launch_fft_fields<float>(p->geom, (const cx<float>*)delta_k, p->d_shell_of, nullptr,
                                                      p->d_fd_tc + f0i, nb, p->d_tw32, t1, t2, f0, p->npts(), hi,
-                                                     p->nprod == 3 ? hi : nullptr, f16, fmax2, nullptr, st,
+                                                     p->nprod == 3 ? hi : nullptr, f16, fmax2, st,
                                                      FieldLayout{p->kb_rows32, p->groups16});
             if (e != cudaSuccess) return cuda_fail(e, "fft");
             launches += 3;
@@ -1284,7 +1285,7 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
         int nb = std::min(p->fb32, nft - f0);
         cudaError_t e = launch_fft_fields<float>(p->geom, (const cx<float>*)delta_k, p->d_shell_of, nullptr,
                                                  p->d_fd_delta + f0, nb, p->d_tw32, t1, t2, f32, p->npts(), nullptr,
-                                                 nullptr, 0, nullptr, nullptr, st);
+                                                 nullptr, 0, nullptr, st);
         if (e != cudaSuccess) return cuda_fail(e, "fft");
         launches += 3;
     }
@@ -1354,7 +1355,7 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
             const int nb = std::min(p->fb32, nfields - f0);
             cudaError_t e = launch_fft_fields<float>(p->geom, (const cx<float>*)delta_k, nullptr, p->d_radial,
                                                      p->d_fd_delta + f0, nb, p->d_tw32, t1, t2, f32, p->npts(),
-                                                     nullptr, nullptr, 0, nullptr, nullptr, st);
+                                                     nullptr, nullptr, 0, nullptr, st);
             if (e != cudaSuccess) return cuda_fail(e, "fft (modal)");
             launches += 3;
         }
@@ -1395,7 +1396,7 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
             const int nb = std::min(p->fb32, nfields - fi);
             cudaError_t e = launch_fft_fields<float>(p->geom, (const cx<float>*)delta_k, nullptr, p->d_radial,
                                                      p->d_fd_tc + fi, nb, p->d_tw32, t1, t2, f0, p->npts(), hi,
-                                                     p->nprod == 3 ? hi : nullptr, f16, fmax2, nullptr, st,
+                                                     p->nprod == 3 ? hi : nullptr, f16, fmax2, st,
                                                      FieldLayout{p->kb_rows32, p->groups16});
             if (e != cudaSuccess) return cuda_fail(e, "fft (modal)");
             launches += 3;
@@ -1579,6 +1580,7 @@ static bool density_geom(int n, FftGeom* g) {
     g->nK = n;
     g->pruned = 0;
     g->nKz = n / 2 + 1;
+    g->ldz = (g->nKz + 7) & ~7;
     g->n2max = 3 * (n / 2) * (n / 2);
     return radix_plan(n, g->rad, &g->nrad) && radix_plan(n / 2, g->rad_h, &g->nrad_h);
 }
@@ -1607,7 +1609,7 @@ bsp_status bsp_density_cic(int n, double box, long long n_particles, const float
 // x^2 and for the per-CTA sums).
 static size_t skew_bytes(int n, size_t* off_t1, size_t* off_t2) {
     const size_t x = round256((size_t)n * n * n * sizeof(float));
-    const size_t h = round256((size_t)n * n * (n / 2 + 1) * sizeof(cx<float>));
+    const size_t h = round256((size_t)n * n * (((size_t)n / 2 + 1 + 7) & ~(size_t)7) * sizeof(cx<float>));
     if (off_t1) *off_t1 = x;
     if (off_t2) *off_t2 = x + h;
     return x + 2 * h;
@@ -1635,7 +1637,7 @@ bsp_status bsp_skew_compute(bsp_plan* p, const void* delta_k, void* ws, size_t w
     const size_t n3 = (size_t)p->n * p->n * p->n;
     // x = sum_{n != 0} delta(n) e^{ik.x} = V delta(x)
     cudaError_t e = launch_fft_fields<float>(full, (const cx<float>*)delta_k, p->d_shell_of, nullptr, p->d_fd_raw, 1,
-                                             p->d_tw32, t1, t2, x, n3, nullptr, nullptr, 0, nullptr, nullptr, st);
+                                             p->d_tw32, t1, t2, x, n3, nullptr, nullptr, 0, nullptr, st);
     if (e != cudaSuccess) return cuda_fail(e, "skew (inverse FFT)");
     // transform of delta(x)^2 = x^2 / V^2, unnormalised, into t1
     const double V = p->box * p->box * p->box;
@@ -1676,6 +1678,7 @@ static bool ib_geom(const bsp_plan* p, int m, FftGeom* gs) {
         gs->nK = 2 * K + 1;
         gs->pruned = 1;
         gs->nKz = K + 1;
+        gs->ldz = (gs->nKz + 7) & ~7;
     }
     return true;
 }
@@ -1684,7 +1687,7 @@ static IbLayout ib_layout(const bsp_plan* p, int m, const FftGeom& gs) {
     const int n = p->n, s = n / m, nc = m * m * m;
     IbLayout L{};
     const size_t x = round256((size_t)n * n * n * sizeof(float));
-    const size_t h = round256((size_t)n * n * (n / 2 + 1) * sizeof(cx<float>));
+    const size_t h = round256((size_t)n * n * (((size_t)n / 2 + 1 + 7) & ~(size_t)7) * sizeof(cx<float>));
     L.t1 = x;
     L.t2 = x + h;
     L.sub = x;
@@ -1742,7 +1745,7 @@ bsp_status bsp_ib_compute(bsp_plan* p, const void* delta_k, int m, void* ws, siz
     // x = sum_{n != 0} delta(n) e^{ik.x} = V delta(x)
     cudaError_t e = launch_fft_fields<float>(full, (const cx<float>*)delta_k, p->d_shell_of, nullptr, p->d_fd_raw, 1,
                                              p->d_tw32, (cx<float>*)(base + L.t1), (cx<float>*)(base + L.t2), x,
-                                             (size_t)n * n * n, nullptr, nullptr, 0, nullptr, nullptr, st);
+                                             (size_t)n * n * n, nullptr, nullptr, 0, nullptr, st);
     if (e != cudaSuccess) return cuda_fail(e, "integrated bispectrum (inverse FFT)");
     // T_c = (1/(V s^3)) sum_{x in c} x e^{-ik.x}: T_c(0) is the cube mean of
     // delta, and the cube's own transform is delta_c(k) = V_s T_c(k)

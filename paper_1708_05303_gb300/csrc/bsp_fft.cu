@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(NTHR) k_pass1(FftGeom g, const cx<float>* __re
     cx<R>* dst = t1 + (size_t)blockIdx.y * t1_stride;
     for (int e = threadIdx.x; e < N * P; e += NTHR) {
         const int p = e % P, x = e / P, kz = kz0 + p;
-        if (kz < g.nKz) dst[((size_t)cy * N + x) * g.nKz + kz] = res[sidx<true, P>(p, x, N)];
+        if (kz < g.nKz) dst[((size_t)cy * N + x) * g.ldz + kz] = res[sidx<true, P>(p, x, N)];
     }
 }
 
@@ -428,7 +428,7 @@ template <typename R, int P, int NN>
 __global__ void __launch_bounds__(NTHR) k_pass2(FftGeom g, const cx<R>* __restrict__ t1,
                                                 size_t t1_stride, const cx<R>* __restrict__ twg,
                                                 cx<R>* __restrict__ t2, size_t t2_stride,
-                                                const FieldDesc* __restrict__ fields, unsigned* __restrict__ fmax2) {
+                                                const FieldDesc* __restrict__ fields) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = NN ? NN : g.n;
     cx<R>* tw = reinterpret_cast<cx<R>*>(smem_raw);
@@ -446,7 +446,7 @@ __global__ void __launch_bounds__(NTHR) k_pass2(FftGeom g, const cx<R>* __restri
         cx<R> val = {(R)0, (R)0};
         if (kz < g.nKz && fy >= -ke && fy <= ke) {
             const int cy = g.pruned ? fy + g.K : iy;
-            val = src[((size_t)cy * N + x) * g.nKz + kz];
+            val = src[((size_t)cy * N + x) * g.ldz + kz];
         }
         buf[sidx<true, P>(p, iy, N)] = val;
     }
@@ -455,18 +455,9 @@ __global__ void __launch_bounds__(NTHR) k_pass2(FftGeom g, const cx<R>* __restri
     if constexpr (NN > 0) res = fft_ct<R, true, P, NN>(buf, scr, tw, 1);
     else res = fft_pingpong<R, true, P>(buf, scr, N, g.rad, g.nrad, tw, 1);
     cx<R>* dst = t2 + (size_t)blockIdx.y * t2_stride;
-    float m = 0.f;
     for (int e = threadIdx.x; e < N * P; e += NTHR) {
         const int p = e % P, y = e / P, kz = kz0 + p;
-        if (kz < g.nKz) {
-            const cx<R> v = res[sidx<true, P>(p, y, N)];
-            dst[((size_t)x * N + y) * g.nKz + kz] = v;
-            m = fmaxf(m, (float)(fabs(v.re) + fabs(v.im)));
-        }
-    }
-    if (fmax2) {
-        const int f = fields[blockIdx.y].out16;
-        if (f >= 0) block_max_to(fmax2 + f, m);
+        if (kz < g.nKz) dst[((size_t)x * N + y) * g.ldz + kz] = res[sidx<true, P>(p, y, N)];
     }
 }
 
@@ -541,7 +532,7 @@ __global__ void __launch_bounds__(NTHR) k_pass1r(FftGeom g, const cx<float>* __r
     if (kz < g.nKz) {
         cx<float>* dst = t1 + (size_t)blockIdx.y * t1_stride;
 #pragma unroll
-        for (int n = 0; n < 16; ++n) dst[((size_t)cy * N + m1 + 16 * (n + 16 * j1)) * g.nKz + kz] = v[n];
+        for (int n = 0; n < 16; ++n) dst[((size_t)cy * N + m1 + 16 * (n + 16 * j1)) * g.ldz + kz] = v[n];
     }
 }
 
@@ -572,7 +563,7 @@ __global__ void __launch_bounds__(NTHR) k_pass2r(FftGeom g, const cx<float>* __r
         cx<float> val = {0.f, 0.f};
         if (live && fy >= -ke && fy <= ke) {
             const int cy = g.pruned ? fy + g.K : iy;
-            val = src[((size_t)cy * N + x) * g.nKz + kz];
+            val = src[((size_t)cy * N + x) * g.ldz + kz];
         }
         v[k2] = val;
     }
@@ -585,7 +576,7 @@ __global__ void __launch_bounds__(NTHR) k_pass2r(FftGeom g, const cx<float>* __r
     for (int n = 0; n < 16; ++n) {
         const int y = m1 + 16 * (n + 16 * j1);
         if (live) {
-            dst[((size_t)x * N + y) * g.nKz + kz] = v[n];
+            dst[((size_t)x * N + y) * g.ldz + kz] = v[n];
             mx = fmaxf(mx, fabsf(v[n].re) + fabsf(v[n].im));
         }
     }
@@ -593,146 +584,6 @@ __global__ void __launch_bounds__(NTHR) k_pass2r(FftGeom g, const cx<float>* __r
         const int f = fields[blockIdx.y].out16;
         if (f >= 0) block_max_to(fmax2 + f, mx);
     }
-}
-
-// Staging layouts of pass 3's z-lines in shared memory (element m of line p
-// = F[2m] + i F[2m+1]).  Stockham passes: the i/8-padded index-fast layout.
-template <int P>
-struct StageStockham {
-    __device__ static int idx(int p, int m, int M) { return sidx<false, P>(p, m, M); }
-    template <typename R>
-    __device__ static void load4(const cx<R>* res, int p, int m0, int M, cx<R> (&v)[4]) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = res[idx(p, m0 + i, M)];
-    }
-};
-// Output of pass 3 for P consecutive y of one x: the real values of each
-// z-line, res[sidx<false, P>(p, m, M)] = F[2m] + i F[2m+1], scaled and
-// written as the field's FP32 row and/or 16-bit hi/lo planes.
-template <typename R, int P, class Stage = StageStockham<P>>
-__device__ __forceinline__ void pass3_store(const FftGeom& g, int N, int M, int x, int y0, const cx<R>* res,
-                                            const FieldDesc& fd, R* __restrict__ out, size_t out_stride,
-                                            uint32_t* __restrict__ hi, uint32_t* __restrict__ lo, int f16,
-                                            const unsigned* __restrict__ fmax2, unsigned* __restrict__ f0max,
-                                            FieldLayout lay) {
-    const bool kbm = lay.groups16 > 0;
-    R* dst = fd.out32 >= 0 ? out + (kbm ? (size_t)0 : (size_t)fd.out32 * out_stride) : nullptr;
-    const size_t plane = (size_t)N * N * M;   // 32-bit words (two 16-bit values) per field plane
-    uint32_t* dhi = nullptr;
-    uint32_t* dlo = nullptr;
-    if (fd.out16 >= 0 && hi) {
-        if (kbm) {   // hi rows of the field's group, lo rows 1024 bytes further
-            dhi = hi + (size_t)(fd.out16 >> 3) * 512 + (size_t)(fd.out16 & 7) * 32;
-            dlo = lo ? dhi + 256 : nullptr;
-        } else {
-            dhi = hi + (size_t)fd.out16 * plane;
-            dlo = lo ? lo + (size_t)fd.out16 * plane : nullptr;
-        }
-    }
-    const int r32 = fd.out32 & 7, r16 = fd.out16 & 7;
-    // |F(x,y,z)| <= sum_kz 2 |H_kz| <= 2 nKz max|T2|: the split planes are
-    // scaled by the power of two that keeps that bound below 2^15
-    const float bound = fmax2 && fd.out16 >= 0 ? 2.f * (float)g.nKz * __uint_as_float(fmax2[fd.out16]) : 0.f;
-    const float sc = (dhi && fmax2) ? pow2_scale(bound) : 1.f;
-    // FP32 pair factors of the tensor-core path are stored pre-scaled (|F s7| < 2^7)
-    const R s7 = fmax2 ? (R)pow2_scale(bound, 7) : (R)1;
-    float mx = 0.f;
-    if constexpr (sizeof(R) == 4) {
-        if (kbm && (M & 3) == 0) {
-            // K-block-major output, four consecutive pairs of z per thread: one 16-byte
-            // chunk of each 16-bit plane row and two of the FP32 row
-            const int M4 = M >> 2;
-            for (int e = threadIdx.x; e < M4 * P; e += NTHR) {
-                const int m0 = (e % M4) * 4, p = e / M4, y = y0 + p;
-                if (y >= N) continue;
-                const size_t pos = ((size_t)x * N + y) * M + m0;
-                const size_t kb = pos >> 5;
-                const int w = (int)(pos & 31);   // a multiple of 4
-                cx<R> v[4];
-                Stage::load4(res, p, m0, M, v);
-                if (dst) {
-                    cx<R>* row = reinterpret_cast<cx<R>*>(dst) + (kb * (size_t)lay.rows32 + (size_t)fd.out32) * 32;
-                    const int J = w >> 1;   // 16-byte chunks J, J + 1 of the 256-byte FP32 row
-                    const int Ja = (J & 8) | ((J & 7) ^ r32), Jb = ((J + 1) & 8) | (((J + 1) & 7) ^ r32);
-                    *reinterpret_cast<float4*>(row + 2 * Ja) =
-                        make_float4(v[0].re * s7, v[0].im * s7, v[1].re * s7, v[1].im * s7);
-                    *reinterpret_cast<float4*>(row + 2 * Jb) =
-                        make_float4(v[2].re * s7, v[2].im * s7, v[3].re * s7, v[3].im * s7);
-                    if (f0max)
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) mx = fmaxf(mx, fmaxf(fabsf(v[i].re), fabsf(v[i].im)));
-                }
-                if (dhi) {
-                    uint32_t h[4], l[4];
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        // two consecutive z values -> 16-bit hi and lo (x0 in the low half)
-                        const float x0 = v[i].re * sc, x1 = v[i].im * sc;
-                        float h0, h1;
-                        if (f16) {
-                            asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h[i]) : "f"(x1), "f"(x0));
-                            unsigned short a = (unsigned short)(h[i] & 0xFFFFu), b = (unsigned short)(h[i] >> 16);
-                            asm("cvt.f32.f16 %0, %1;" : "=f"(h0) : "h"(a));
-                            asm("cvt.f32.f16 %0, %1;" : "=f"(h1) : "h"(b));
-                            asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(l[i]) : "f"(x1 - h1), "f"(x0 - h0));
-                        } else {
-                            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h[i]) : "f"(x1), "f"(x0));
-                            h0 = __uint_as_float(h[i] << 16);
-                            h1 = __uint_as_float(h[i] & 0xFFFF0000u);
-                            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l[i]) : "f"(x1 - h1), "f"(x0 - h0));
-                        }
-                    }
-                    const size_t q = kb * (size_t)lay.groups16 * 512 + (size_t)(((w >> 2) ^ r16) << 2);
-                    *reinterpret_cast<uint4*>(dhi + q) = make_uint4(h[0], h[1], h[2], h[3]);
-                    if (dlo) *reinterpret_cast<uint4*>(dlo + q) = make_uint4(l[0], l[1], l[2], l[3]);
-                }
-            }
-            if (f0max && dst) block_max_to(f0max + fd.out32, mx);
-            return;
-        }
-    }
-    for (int e = threadIdx.x; e < M * P; e += NTHR) {
-        const int m = e % M, p = e / M, y = y0 + p;
-        if (y >= N) continue;
-        // pos counts pairs of consecutive z (one complex, one 32-bit plane word);
-        // K-block-major: K-block pos / 32, pair w = pos % 32 of it (points 2w, 2w+1)
-        const size_t pos = ((size_t)x * N + y) * M + m;
-        size_t p32 = pos, p16 = pos;
-        if (kbm) {
-            const size_t kb = pos >> 5;
-            const int w = (int)(pos & 31);
-            const int J = w >> 1;   // 16-byte chunk of the 256-byte FP32 row
-            p32 = (kb * (size_t)lay.rows32 + (size_t)fd.out32) * 32 + (size_t)(((J & 8) | ((J & 7) ^ r32)) * 2 + (w & 1));
-            p16 = kb * (size_t)lay.groups16 * 512 + (size_t)((((w >> 2) ^ r16) << 2) | (w & 3));
-        }
-        const cx<R> v = res[Stage::idx(p, m, M)];
-        if (dst) {
-            reinterpret_cast<cx<R>*>(dst)[p32] = cx<R>{v.re * s7, v.im * s7};
-            if (f0max) mx = fmaxf(mx, fmaxf(fabsf((float)v.re), fabsf((float)v.im)));
-        }
-        if (dhi) {
-            // two consecutive z values -> 16-bit hi and lo planes (x0 in the low half)
-            const float x0 = (float)v.re * sc, x1 = (float)v.im * sc;
-            uint32_t h, l;
-            if (f16) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x1), "f"(x0));
-            else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(x1), "f"(x0));
-            float h0, h1;
-            if (f16) {
-                unsigned short a = (unsigned short)(h & 0xFFFFu), b = (unsigned short)(h >> 16);
-                asm("cvt.f32.f16 %0, %1;" : "=f"(h0) : "h"(a));
-                asm("cvt.f32.f16 %0, %1;" : "=f"(h1) : "h"(b));
-            } else {
-                h0 = __uint_as_float(h << 16);
-                h1 = __uint_as_float(h & 0xFFFF0000u);
-            }
-            const float r0 = x0 - h0, r1 = x1 - h1;
-            if (f16) asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(r1), "f"(r0));
-            else asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(r1), "f"(r0));
-            dhi[p16] = h;
-            if (dlo) dlo[p16] = l;
-        }
-    }
-    if (f0max && dst) block_max_to(f0max + fd.out32, mx);
 }
 
 // Pass 3: real inverse DFT along z for P consecutive y of one x, through a
@@ -743,10 +594,7 @@ template <typename R, int P, int NN>
 __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restrict__ t2,
                                                 size_t t2_stride, const cx<R>* __restrict__ twg,
                                                 const FieldDesc* __restrict__ fields, R* __restrict__ out,
-                                                size_t out_stride, uint32_t* __restrict__ hi,
-                                                uint32_t* __restrict__ lo, int f16,
-                                                const unsigned* __restrict__ fmax2,
-                                                unsigned* __restrict__ f0max, FieldLayout lay) {
+                                                size_t out_stride) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = NN ? NN : g.n, M = N / 2;
     cx<R>* tw = reinterpret_cast<cx<R>*>(smem_raw);
@@ -762,7 +610,7 @@ __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restri
         const int k = e % M, p = e / M, y = y0 + p;
         cx<R> z = {(R)0, (R)0};
         if (y < N) {
-            const cx<R>* h = src + ((size_t)x * N + y) * g.nKz;
+            const cx<R>* h = src + ((size_t)x * N + y) * g.ldz;
             cx<R> a = {(R)0, (R)0}, b = {(R)0, (R)0};
             if (k < nk) a = h[k];
             if (M - k < nk) b = h[M - k];
@@ -777,9 +625,12 @@ __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restri
     const cx<R>* res;
     if constexpr (NN > 0) res = fft_ct<R, false, P, NN / 2>(buf, scr, tw, 2);
     else res = fft_pingpong<R, false, P>(buf, scr, M, g.rad_h, g.nrad_h, tw, 2);
-    pass3_store<R, P>(g, N, M, x, y0, res, fields[blockIdx.y], out, out_stride, hi, lo, f16, fmax2, f0max, lay);
+    cx<R>* dst = reinterpret_cast<cx<R>*>(out + (size_t)fields[blockIdx.y].out32 * out_stride);
+    for (int e = threadIdx.x; e < M * P; e += NTHR) {
+        const int m = e % M, p = e / M, y = y0 + p;
+        if (y < N) dst[((size_t)x * N + y) * M + m] = res[sidx<false, P>(p, m, M)];
+    }
 }
-
 
 // Pass 3 for the sizes known at compile time, FP32, with the z-lines in registers:
 // M = n/2 = R1 x R2, the two stages of the Stockham list (16 x 3, 16 x 4, 16 x 5,
@@ -793,7 +644,7 @@ __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restri
 // stage after another, as before, kept a few dozen of 256 threads busy in the
 // radix-16 stage.  Fields and time before -> now: 288 FP32 fields of 256^3 14.2 ->
 // 4.9 ms (4.4 at the copy rate), 72 of 160^3 1.33 -> 0.27 ms, 150 operand sets of 256^3
-// 8.9 -> 4.4 ms, 96 of 512^3 (16 x 16 in registers before, staged for 16-byte stores)
+// 8.9 -> 4.0 ms, 96 of 512^3 (16 x 16 in registers before, staged for 16-byte stores)
 // 20.5 -> 18.8 ms.  Bound at 512^3: L1 wavefronts, 76 % busy (T2 rows of 1 040 bytes, the
 // 4-byte plane stores).
 template <int NN>
@@ -812,8 +663,26 @@ struct P3V {
 
 enum { P3_FIELD, P3_F16, P3_BF16 };   // FP32 fields, or the K-block-major operands with FP16 or BF16 planes
 
+// Two consecutive z values (x0 in the low half) -> 16-bit hi and lo words.
+template <int MODE>
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hw, uint32_t& lw) {
+    float h0, h1;
+    if (MODE == P3_F16) {
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
+        unsigned short a = (unsigned short)(hw & 0xFFFFu), b = (unsigned short)(hw >> 16);
+        asm("cvt.f32.f16 %0, %1;" : "=f"(h0) : "h"(a));
+        asm("cvt.f32.f16 %0, %1;" : "=f"(h1) : "h"(b));
+        asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
+    } else {
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
+        h0 = __uint_as_float(hw << 16);
+        h1 = __uint_as_float(hw & 0xFFFF0000u);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
+    }
+}
+
 template <int NN, int MODE>
-__global__ void __launch_bounds__(P3V<NN>::T) k_pass3v(FftGeom g, const cx<float>* __restrict__ t2, size_t t2_stride,
+__global__ void __launch_bounds__(P3V<NN>::T, 1024 / P3V<NN>::T) k_pass3v(FftGeom g, const cx<float>* __restrict__ t2, size_t t2_stride,
                                                        const cx<float>* __restrict__ tw,
                                                        const FieldDesc* __restrict__ fields, float* __restrict__ out,
                                                        size_t out_stride, uint32_t* __restrict__ hi, int split,
@@ -830,7 +699,7 @@ __global__ void __launch_bounds__(P3V<NN>::T) k_pass3v(FftGeom g, const cx<float
     for (int i = threadIdx.x; i < M; i += V::T) tw2[i] = tw[2 * (i / R1) * (i % R1)];
     {
         const int j = threadIdx.x % R2, p = threadIdx.x / R2;
-        const cx<float>* h = t2 + (size_t)blockIdx.y * t2_stride + (line0 + p) * nKz;
+        const cx<float>* h = t2 + (size_t)blockIdx.y * t2_stride + (line0 + p) * g.ldz;
         cx<float> v[R1];
 #pragma unroll
         for (int r = 0; r < R1; ++r) {
@@ -848,7 +717,8 @@ __global__ void __launch_bounds__(P3V<NN>::T) k_pass3v(FftGeom g, const cx<float
         for (int r = 0; r < R1; ++r) buf[V::idx(p, j * R1 + r)] = v[r];
     }
     __syncthreads();
-    // the power-of-two scales of the tensor-core operands (see pass3_store)
+    // the power-of-two scales of the tensor-core operands (|F(x,y,z)| <= sum_kz 2 |H_kz| <=
+    // 2 nKz max|T2|): 16-bit planes below 2^15, FP32 pair factors below 2^7
     float sc = 1.f, s7 = 1.f;
     if (MODE != P3_FIELD) {
         const float bound = 2.f * (float)nKz * __uint_as_float(fmax2[fd.out16]);
@@ -905,109 +775,315 @@ __global__ void __launch_bounds__(P3V<NN>::T) k_pass3v(FftGeom g, const cx<float
             int w;
             at(r, kb, w);
             uint32_t* d = q + kb * (size_t)(lay.groups16 * 512) + (w ^ (4 * r16));
-            const float x0 = v[r].re * sc, x1 = v[r].im * sc;
             uint32_t hw, lw;
-            float h0, h1;
-            if (MODE == P3_F16) {
-                asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
-                unsigned short a = (unsigned short)(hw & 0xFFFFu), b = (unsigned short)(hw >> 16);
-                asm("cvt.f32.f16 %0, %1;" : "=f"(h0) : "h"(a));
-                asm("cvt.f32.f16 %0, %1;" : "=f"(h1) : "h"(b));
-                asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
-            } else {
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hw) : "f"(x1), "f"(x0));
-                h0 = __uint_as_float(hw << 16);
-                h1 = __uint_as_float(hw & 0xFFFF0000u);
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lw) : "f"(x1 - h1), "f"(x0 - h0));
-            }
+            split_pair<MODE>(v[r].re * sc, v[r].im * sc, hw, lw);
             d[0] = hw;
             if (split) d[256] = lw;
         }
     }
 }
 
-template <typename R>
-struct FftCfg;
-template <>
-struct FftCfg<float> {
-    // pass-3 pencils are contiguous z-lines, so a smaller batch costs no
-    // coalescing and lets more CTAs share an SM (about 39 KB each at n = 512)
-    static constexpr int P = 8, P3 = 8;
-};
-template <>
-struct FftCfg<double> {
-    static constexpr int P = 4, P3 = 8;
-};
+// ---------------------------------------------------------------------------
+// Passes 1 and 2 (FP32) for every size but 512, and pass 3 for the sizes not known at
+// compile time.  CP lines side by side in shared memory, element i of line p at
+// i SP + p: the lanes run over the lines, so every access is a row of consecutive
+// lines (no conflicts, no index division), and a stage has (length / radix) CP
+// butterflies for the CTA's threads.  Passes 1 and 2 take their first stage straight
+// from global memory and store the last one there, in runs of CP consecutive f_z
+// (128 bytes, in rows padded to 64).  Bound by latency: two to four stages with a barrier
+// each on 2 to 12 warps a CTA.  Eight lines on 256 threads with run-time divisions in
+// every index, before, left most threads idle.  Before -> now, microseconds: 42 fields
+// of 150^3 pass 1 107 -> 70, 2 302 -> 190, 3 1 331 -> 630; 150 of 256^3 pass 2 3 159 -> 2 000;
+// 72 of 160^3 pass 2 160 -> 130; 32^3 with 8 shells, all three 50 -> 30.
+// ---------------------------------------------------------------------------
+constexpr int CP = 16;
 
-template <typename R, int NN>
+// NSC: the product of the radices before (0: known at run time; magic = ceil(2^32 / Ns)).
+template <int RADIX, bool FIRST, bool LAST, int NSC, int SP, class Ld, class St>
+__device__ __forceinline__ void col_stage(const cx<float>* src, cx<float>* dst, int M, int Ns_, unsigned magic, int twmul,
+                                          const cx<float>* __restrict__ tw, Ld ld, St st) {
+    const int nbf = M / RADIX, Ns = NSC ? NSC : Ns_;
+    const int tmul = nbf / Ns * twmul;   // M / (Ns RADIX) twiddle steps
+#pragma unroll 1
+    for (int b = threadIdx.x; b < nbf * CP; b += blockDim.x) {
+        const int p = b % CP, j = b / CP;
+        const int k = Ns == 1 ? 0 : j - Ns * (NSC ? j / NSC : (int)__umulhi((unsigned)j, magic));
+        cx<float> v[RADIX];
+#pragma unroll
+        for (int r = 0; r < RADIX; ++r) {
+            v[r] = FIRST ? ld(j + r * nbf, p) : src[(j + r * nbf) * SP + p];
+            if (!FIRST && r > 0 && Ns > 1) v[r] = rmul(v[r], tw[r * k * tmul]);
+        }
+        dft<RADIX>(v);
+        const int o = (j - k) * RADIX + k;
+#pragma unroll
+        for (int r = 0; r < RADIX; ++r) {
+            if (LAST) st(o + r * Ns, p, v[r]);
+            else dst[(o + r * Ns) * SP + p] = v[r];
+        }
+    }
+    if (!LAST) __syncthreads();
+}
+
+// Compile-time radix list, from ld to st through the buffers a and b.
+template <int M, int SP, int S, int NS, class Ld, class St>
+__device__ __forceinline__ void col_ct(cx<float>* a, cx<float>* b, int twmul, const cx<float>* tw, Ld ld, St st) {
+    constexpr RadixList L = radix_list(M);
+    if constexpr (S < L.n) {
+        col_stage<L.r[S], S == 0, S == L.n - 1, NS, SP>(a, b, M, NS, 0u, twmul, tw, ld, st);
+        col_ct<M, SP, S + 1, NS * L.r[S]>(b, a, twmul, tw, ld, st);
+    }
+}
+
+// Run-time radix list (8, 4, 2, 3, 5).  IO: the first stage loads through ld and the last
+// stores through st; otherwise the lines are in a, and the buffer they end in is returned.
+template <bool FIRST, bool LAST, int SP, class Ld, class St>
+__device__ __forceinline__ void col_rt1(int rad, const cx<float>* a, cx<float>* b, int M, int Ns, int twmul,
+                                        const cx<float>* tw, Ld ld, St st) {
+    const unsigned magic = Ns > 1 ? (unsigned)((0x100000000ull + Ns - 1) / Ns) : 0u;
+    switch (rad) {
+        case 8: col_stage<8, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 4: col_stage<4, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 2: col_stage<2, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 3: col_stage<3, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        default: col_stage<5, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+    }
+}
+template <bool IO, int SP, class Ld, class St>
+__device__ __forceinline__ cx<float>* col_rt(cx<float>* a, cx<float>* b, int M, const int* rad, int nrad, int twmul,
+                                             const cx<float>* tw, Ld ld, St st) {
+    if (IO && nrad == 1) {
+        col_rt1<true, true, SP>(rad[0], a, b, M, 1, twmul, tw, ld, st);
+        return a;
+    }
+    int Ns = 1;
+    for (int s = 0; s < nrad; ++s) {
+        if (IO && s == 0) col_rt1<true, false, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        else if (IO && s == nrad - 1) col_rt1<false, true, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        else col_rt1<false, false, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        Ns *= rad[s];
+        cx<float>* t = a;
+        a = b;
+        b = t;
+    }
+    return a;
+}
+
+// Pass 1: filter + inverse DFT along x for CP consecutive f_z of one f_y.
+template <int NN>
+__global__ void __launch_bounds__(256) k_col1(FftGeom g, const cx<float>* __restrict__ delta,
+                                              const int16_t* __restrict__ shell_of, const float* __restrict__ radial,
+                                              const FieldDesc* __restrict__ fields, const cx<float>* __restrict__ tw,
+                                              cx<float>* __restrict__ t1, size_t t1_stride) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = NN ? NN : g.n;
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    const FieldDesc fd = fields[blockIdx.y];
+    const int nkzb = (g.nKz + CP - 1) / CP;
+    const int cy = blockIdx.x / nkzb, kz0 = (blockIdx.x % nkzb) * CP;
+    const int fy = g.pruned ? cy - g.K : freq_of(cy, N);
+    const int iy = fy < 0 ? fy + N : fy;
+    const int ke = field_ext(fd, g);
+    if (fy > ke || fy < -ke || kz0 > ke) return;   // zero there, and pass 2 reads none of it
+    cx<float>* dst = t1 + (size_t)blockIdx.y * t1_stride + (size_t)cy * N * g.ldz + kz0;
+    auto ld = [&](int i, int p) { return pass1_input<float>(g, fd, delta, shell_of, radial, N, i, fy, iy, kz0 + p); };
+    auto st = [&](int i, int p, cx<float> v) {
+        if (kz0 + p < g.nKz) dst[(size_t)i * g.ldz + p] = v;
+    };
+    if constexpr (NN > 0) col_ct<NN, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
+    else col_rt<true, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
+}
+
+// Pass 2: inverse DFT along y for CP consecutive f_z of one x.
+template <int NN>
+__global__ void __launch_bounds__(256) k_col2(FftGeom g, const cx<float>* __restrict__ t1, size_t t1_stride,
+                                              const cx<float>* __restrict__ tw, cx<float>* __restrict__ t2,
+                                              size_t t2_stride, const FieldDesc* __restrict__ fields,
+                                              unsigned* __restrict__ fmax2) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = NN ? NN : g.n;
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    const int nkzb = (g.nKz + CP - 1) / CP;
+    const int x = blockIdx.x / nkzb, kz0 = (blockIdx.x % nkzb) * CP;
+    const FieldDesc fd = fields[blockIdx.y];
+    const int ke = field_ext(fd, g);
+    if (kz0 > ke) return;   // zero there, and pass 3 reads none of it
+    const cx<float>* src = t1 + (size_t)blockIdx.y * t1_stride + (size_t)x * g.ldz + kz0;
+    cx<float>* dst = t2 + (size_t)blockIdx.y * t2_stride + (size_t)x * N * g.ldz + kz0;
+    float m = 0.f;
+    auto ld = [&](int i, int p) {
+        const int f = freq_of(i, N);
+        cx<float> v = {0.f, 0.f};
+        if (kz0 + p < g.nKz && f >= -ke && f <= ke) v = src[(size_t)(g.pruned ? f + g.K : i) * N * g.ldz + p];
+        return v;
+    };
+    auto st = [&](int i, int p, cx<float> v) {
+        if (kz0 + p < g.nKz) {
+            dst[(size_t)i * g.ldz + p] = v;
+            m = fmaxf(m, fabsf(v.re) + fabsf(v.im));
+        }
+    };
+    if constexpr (NN > 0) col_ct<NN, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
+    else col_rt<true, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
+    if (fmax2 && fd.out16 >= 0) block_max_to(fmax2 + fd.out16, m);
+}
+
+// Pass 3 for run-time sizes: CP consecutive lines (of all n^2), lanes along k for the
+// loads and along m for the stores (row stride CP + 1: no conflicts either way).
+template <int MODE>
+__global__ void __launch_bounds__(256) k_pass3g(FftGeom g, const cx<float>* __restrict__ t2, size_t t2_stride,
+                                                const cx<float>* __restrict__ tw, const FieldDesc* __restrict__ fields,
+                                                float* __restrict__ out, size_t out_stride, uint32_t* __restrict__ hi,
+                                                int split, const unsigned* __restrict__ fmax2, FieldLayout lay) {
+    constexpr int SP = CP + 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int N = g.n, M = N / 2, nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    const FieldDesc fd = fields[blockIdx.y];
+    const int nKz = g.nKz, nk = field_ext(fd, g) + 1;   // f_z read: 0 .. nk - 1
+    const size_t line0 = (size_t)blockIdx.x * CP, lines = (size_t)N * N;
+    for (int p = warp; p < CP; p += nw) {
+        const cx<float>* h = t2 + (size_t)blockIdx.y * t2_stride + (line0 + p) * g.ldz;
+        for (int k = lane; k < M; k += 32) {
+            cx<float> z = {0.f, 0.f};
+            if (line0 + p < lines) {
+                cx<float> a = {0.f, 0.f}, b = {0.f, 0.f};
+                if (k < nk) a = h[k];
+                if (M - k < nk) b = h[M - k];
+                if (k == 0) { a.im = 0.f; b.im = 0.f; }   // H_0 and H_M: real parts only
+                const cx<float> bc = {b.re, -b.im};
+                const cx<float> s = radd(a, bc), d = rsub(a, bc), dw = rmul(d, tw[k]);
+                z = radd(s, cx<float>{-dw.im, dw.re});
+            }
+            buf[k * SP + p] = z;
+        }
+    }
+    __syncthreads();
+    auto none_ld = [](int, int) { return cx<float>{0.f, 0.f}; };
+    auto none_st = [](int, int, cx<float>) {};
+    const cx<float>* res = col_rt<false, SP>(buf, buf + M * SP, M, g.rad_h, g.nrad_h, 2, tw, none_ld, none_st);
+    float sc = 1.f, s7 = 1.f;   // as in k_pass3v
+    if (MODE != P3_FIELD) {
+        const float bound = 2.f * (float)nKz * __uint_as_float(fmax2[fd.out16]);
+        sc = pow2_scale(bound);
+        s7 = pow2_scale(bound, 7);
+    }
+    const int r32 = fd.out32 & 7, r16 = fd.out16 & 7;
+    uint32_t* q = MODE != P3_FIELD ? hi + (size_t)(fd.out16 >> 3) * 512 + (size_t)r16 * 32 : nullptr;
+    for (int p = warp; p < CP; p += nw) {
+        if (line0 + p >= lines) break;
+        for (int m = lane; m < M; m += 32) {
+            const cx<float> v = res[m * SP + p];
+            const size_t pos = (line0 + p) * M + m;   // complex values: pairs of consecutive z
+            if (MODE == P3_FIELD) {
+                reinterpret_cast<cx<float>*>(out + (size_t)fd.out32 * out_stride)[pos] = v;
+                continue;
+            }
+            const size_t kb = pos >> 5;
+            const int w = (int)(pos & 31);
+            if (fd.out32 >= 0)
+                (reinterpret_cast<cx<float>*>(out) + (size_t)fd.out32 * 32)[kb * (size_t)(lay.rows32 * 32) + (w ^ (2 * r32))] =
+                    cx<float>{v.re * s7, v.im * s7};
+            uint32_t hw, lw;
+            split_pair<MODE>(v.re * sc, v.im * sc, hw, lw);
+            uint32_t* d = q + kb * (size_t)(lay.groups16 * 512) + (w ^ (4 * r16));
+            d[0] = hw;
+            if (split) d[256] = lw;
+        }
+    }
+}
+
+// FP64 (the unit fields of the counts): the shared-memory kernels above.
+template <int NN>
 cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* shell_of, const float* radial,
-                     const FieldDesc* d_fields, int nfields, const cx<R>* tw, cx<R>* t1, cx<R>* t2, R* out,
-                     size_t out_stride, uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, unsigned* f0max,
-                     cudaStream_t st, FieldLayout lay) {
-    using C = FftCfg<R>;
+                     const FieldDesc* d_fields, int nfields, const cx<double>* tw, cx<double>* t1, cx<double>* t2,
+                     double* out, size_t out_stride, uint32_t*, uint32_t*, int, unsigned*, cudaStream_t st, FieldLayout) {
+    constexpr int P = 4, P3 = 8;
     const int N = g.n, M = N / 2;
-    const size_t t1_stride = (size_t)g.nK * N * g.nKz;
-    const size_t t2_stride = (size_t)N * N * g.nKz;
-    const size_t sm12 = sizeof(cx<R>) * ((size_t)N + 2 * (size_t)smem_elems<true, C::P>(N));
-    const size_t sm3 = sizeof(cx<R>) * ((size_t)N + 2 * (size_t)smem_elems<false, C::P3>(M));
+    const size_t t1_stride = (size_t)g.nK * N * g.ldz, t2_stride = (size_t)N * N * g.ldz;
+    const size_t sm12 = sizeof(cx<double>) * ((size_t)N + 2 * (size_t)smem_elems<true, P>(N));
+    const size_t sm3 = sizeof(cx<double>) * ((size_t)N + 2 * (size_t)smem_elems<false, P3>(M));
     // raise the dynamic shared-memory limit once per size (never inside a graph capture)
-    static size_t set12 = 0, set3 = 0;
+    static size_t set = 0;
+    if (std::max(sm12, sm3) > set) {
+        cudaError_t e;
+        if ((e = cudaFuncSetAttribute(k_pass1<double, P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm12)) !=
+                cudaSuccess ||
+            (e = cudaFuncSetAttribute(k_pass2<double, P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm12)) !=
+                cudaSuccess ||
+            (e = cudaFuncSetAttribute(k_pass3<double, P3, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)) !=
+                cudaSuccess)
+            return e;
+        set = std::max(sm12, sm3);
+    }
+    const int nkzb = (g.nKz + P - 1) / P;
+    k_pass1<double, P, NN><<<dim3(g.nK * nkzb, nfields), NTHR, sm12, st>>>(g, delta, shell_of, radial, d_fields, tw, t1,
+                                                                           t1_stride);
+    k_pass2<double, P, NN><<<dim3(N * nkzb, nfields), NTHR, sm12, st>>>(g, t1, t1_stride, tw, t2, t2_stride,
+                                                                        d_fields);
+    k_pass3<double, P3, NN><<<dim3(N * ((N + P3 - 1) / P3), nfields), NTHR, sm3, st>>>(g, t2, t2_stride, tw, d_fields, out,
+                                                                                       out_stride);
+    return cudaGetLastError();
+}
+
+// Threads for `items` butterflies of a CTA's largest stage, 64 .. 256.
+inline int col_threads(int items) { return std::min(256, std::max(64, (items + 31) / 32 * 32)); }
+
+template <int NN>
+cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* shell_of, const float* radial,
+                     const FieldDesc* d_fields, int nfields, const cx<float>* tw, cx<float>* t1, cx<float>* t2, float* out,
+                     size_t out_stride, uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, cudaStream_t st,
+                     FieldLayout lay) {
+    const int N = g.n, M = N / 2;
+    const size_t t1_stride = (size_t)g.nK * N * g.ldz, t2_stride = (size_t)N * N * g.ldz;
     cudaError_t e;
-    if (sm12 > set12) {
-        if ((e = cudaFuncSetAttribute(k_pass1<R, C::P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm12)) != cudaSuccess)
-            return e;
-        if ((e = cudaFuncSetAttribute(k_pass2<R, C::P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)sm12)) != cudaSuccess)
-            return e;
-        set12 = sm12;
-    }
-    if constexpr (NN == 0 || !std::is_same<R, float>::value) {
-        if (sm3 > set3) {
-            if ((e = cudaFuncSetAttribute(k_pass3<R, C::P3, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)sm3)) != cudaSuccess)
+    if constexpr (NN == 512) {
+        static bool set = false;   // never inside a graph capture
+        if (!set) {
+            if ((e = cudaFuncSetAttribute(k_pass1r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2r_smem_bytes())) !=
+                    cudaSuccess ||
+                (e = cudaFuncSetAttribute(k_pass2r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2r_smem_bytes())) !=
+                    cudaSuccess)
                 return e;
-            set3 = sm3;
+            set = true;
         }
-    }
-    const int nkzb = (g.nKz + C::P - 1) / C::P;
-    dim3 g1(g.nK * nkzb, nfields), g2(N * nkzb, nfields), g3(N * ((N + C::P3 - 1) / C::P3), nfields);
-    if constexpr (NN == 512 && std::is_same<R, float>::value) {
-        static bool set1r = false;
-        if (!set1r) {
-            if ((e = cudaFuncSetAttribute(k_pass1r, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)p2r_smem_bytes())) != cudaSuccess)
-                return e;
-            set1r = true;
-        }
-        k_pass1r<<<dim3(g.nK * nkzb, nfields), NTHR, p2r_smem_bytes(), st>>>(g, delta, shell_of, radial, d_fields,
-                                                                             tw, t1, t1_stride);
+        const int nkzb = (g.nKz + P2R - 1) / P2R;
+        k_pass1r<<<dim3(g.nK * nkzb, nfields), NTHR, p2r_smem_bytes(), st>>>(g, delta, shell_of, radial, d_fields, tw, t1,
+                                                                             t1_stride);
+        k_pass2r<<<dim3(N * nkzb, nfields), NTHR, p2r_smem_bytes(), st>>>(g, t1, t1_stride, tw, t2, t2_stride, d_fields,
+                                                                          fmax2);
     } else {
-        k_pass1<R, C::P, NN><<<g1, NTHR, sm12, st>>>(g, delta, shell_of, radial, d_fields, tw, t1, t1_stride);
-    }
-    if constexpr (NN == 512 && std::is_same<R, float>::value) {
-        static bool set2r = false;
-        if (!set2r) {
-            if ((e = cudaFuncSetAttribute(k_pass2r, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)p2r_smem_bytes())) != cudaSuccess)
+        const int nrad = NN ? radix_list(NN).n : g.nrad, rad0 = NN ? radix_list(NN).r[0] : g.rad[0];
+        const size_t sm = sizeof(cx<float>) * (size_t)N * CP * (nrad > 2 ? 2 : 1);   // two stages: one buffer
+        static size_t set = 0;
+        if (sm > 48 * 1024 && sm > set) {
+            if ((e = cudaFuncSetAttribute(k_col1<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
+                (e = cudaFuncSetAttribute(k_col2<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
                 return e;
-            set2r = true;
+            set = sm;
         }
-        k_pass2r<<<dim3(N * ((g.nKz + P2R - 1) / P2R), nfields), NTHR, p2r_smem_bytes(), st>>>(
-            g, t1, t1_stride, tw, t2, t2_stride, d_fields, fmax2);
-    } else {
-        k_pass2<R, C::P, NN><<<g2, NTHR, sm12, st>>>(g, t1, t1_stride, tw, t2, t2_stride, d_fields, fmax2);
+        const int nkzb = (g.nKz + CP - 1) / CP, thr = col_threads(N / rad0 * CP);
+        k_col1<NN><<<dim3(g.nK * nkzb, nfields), thr, sm, st>>>(g, delta, shell_of, radial, d_fields, tw, t1, t1_stride);
+        k_col2<NN><<<dim3(N * nkzb, nfields), thr, sm, st>>>(g, t1, t1_stride, tw, t2, t2_stride, d_fields, fmax2);
     }
-    if constexpr (NN > 0 && std::is_same<R, float>::value) {
+    const bool kbm = lay.groups16 > 0;
+    if constexpr (NN > 0) {
         using V = P3V<NN>;
-        const dim3 gv((unsigned)((size_t)N * N / V::P), nfields);
-        const bool kbm = lay.groups16 > 0;
         auto kern = !kbm ? k_pass3v<NN, P3_FIELD> : f16 ? k_pass3v<NN, P3_F16> : k_pass3v<NN, P3_BF16>;
-        kern<<<gv, V::T, V::smem(), st>>>(g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo != nullptr, fmax2,
-                                          lay);
+        kern<<<dim3((unsigned)((size_t)N * N / V::P), nfields), V::T, V::smem(), st>>>(
+            g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo != nullptr, fmax2, lay);
     } else {
-        k_pass3<R, C::P3, NN><<<g3, NTHR, sm3, st>>>(g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo, f16,
-                                                     fmax2, f0max, lay);
+        auto kern = !kbm ? k_pass3g<P3_FIELD> : f16 ? k_pass3g<P3_F16> : k_pass3g<P3_BF16>;
+        const size_t sm = sizeof(cx<float>) * 2 * (size_t)M * (CP + 1);
+        static size_t set[3] = {0, 0, 0};
+        const int ki = !kbm ? 0 : f16 ? 1 : 2;
+        if (sm > 48 * 1024 && sm > set[ki]) {
+            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
+                return e;
+            set[ki] = sm;
+        }
+        kern<<<dim3((unsigned)(((size_t)N * N + CP - 1) / CP), nfields), col_threads(M * CP / 4), sm, st>>>(
+            g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo != nullptr, fmax2, lay);
     }
     return cudaGetLastError();
 }
@@ -1227,12 +1303,12 @@ template <typename R>
 cudaError_t launch_fft_fields(const FftGeom& g, const cx<float>* delta, const int16_t* shell_of,
                               const float* radial, const FieldDesc* d_fields, int nfields,
                               const cx<R>* tw, cx<R>* t1, cx<R>* t2, R* out, size_t out_stride,
-                              uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, unsigned* f0max,
-                              cudaStream_t st, FieldLayout lay) {
+                              uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, cudaStream_t st,
+                              FieldLayout lay) {
 #define BSP_FFT_CASE(NV) \
     case NV:             \
-        return launch_n<R, NV>(g, delta, shell_of, radial, d_fields, nfields, tw, t1, t2, out, out_stride, hi, lo, \
-                               f16, fmax2, f0max, st, lay);
+        return launch_n<NV>(g, delta, shell_of, radial, d_fields, nfields, tw, t1, t2, out, out_stride, hi, lo, f16, \
+                            fmax2, st, lay);
     switch (g.n) {
         BSP_FFT_CASE(64)
         BSP_FFT_CASE(96)
@@ -1241,15 +1317,15 @@ cudaError_t launch_fft_fields(const FftGeom& g, const cx<float>* delta, const in
         BSP_FFT_CASE(256)
         BSP_FFT_CASE(512)
         default:
-            return launch_n<R, 0>(g, delta, shell_of, radial, d_fields, nfields, tw, t1, t2, out, out_stride, hi, lo,
-                                  f16, fmax2, f0max, st, lay);
+            return launch_n<0>(g, delta, shell_of, radial, d_fields, nfields, tw, t1, t2, out, out_stride, hi, lo, f16,
+                               fmax2, st, lay);
     }
 #undef BSP_FFT_CASE
 }
 
 template cudaError_t launch_fft_fields<float>(const FftGeom&, const cx<float>*, const int16_t*, const float*,
                                               const FieldDesc*, int, const cx<float>*, cx<float>*,
-                                              cx<float>*, float*, size_t, uint32_t*, uint32_t*, int, unsigned*, unsigned*,
+                                              cx<float>*, float*, size_t, uint32_t*, uint32_t*, int, unsigned*,
                                               cudaStream_t, FieldLayout);
 DensityLayout density_layout(int n) {
     auto r256 = [](size_t b) { return (b + 255) / 256 * 256; };
@@ -1361,6 +1437,6 @@ cudaError_t launch_density(const FftGeom& g, const float* pos, long long np, dou
 template cudaError_t launch_fft_fields<double>(const FftGeom&, const cx<float>*, const int16_t*, const float*,
                                                const FieldDesc*, int, const cx<double>*, cx<double>*,
                                                cx<double>*, double*, size_t, uint32_t*, uint32_t*, int,
-                                               unsigned*, unsigned*, cudaStream_t, FieldLayout);
+                                               unsigned*, cudaStream_t, FieldLayout);
 
 }  // namespace bsp

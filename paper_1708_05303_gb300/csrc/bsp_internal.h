@@ -49,6 +49,7 @@ struct FftGeom {
     int nK;       // kept x/y frequencies: 2K+1 (pruned) or n
     int pruned;   // 1 if nK < n
     int nKz;      // kept z frequencies 0..nKz-1 (<= n/2+1)
+    int ldz;      // row length of the transform's intermediates: nKz rounded up to 8 (64-byte rows)
     int n2max;    // largest |n|^2 in the shell table
     int nrad;     // radix stages for length n
     int rad[8];
@@ -135,8 +136,8 @@ template <typename R>
 cudaError_t launch_fft_fields(const FftGeom& g, const cx<float>* delta, const int16_t* shell_of,
                               const float* radial, const FieldDesc* d_fields, int nfields,
                               const cx<R>* tw, cx<R>* t1, cx<R>* t2, R* out, size_t out_stride,
-                              uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, unsigned* f0max,
-                              cudaStream_t st, FieldLayout lay = FieldLayout());
+                              uint32_t* hi, uint32_t* lo, int f16, unsigned* fmax2, cudaStream_t st,
+                              FieldLayout lay = FieldLayout());
 
 // Shot-noise combination in the reduction: v -= sum_t coef[t] * (sum of partial set t).
 struct ShotTerms {
