@@ -799,14 +799,14 @@ __global__ void __launch_bounds__(P3V<NN>::T, 1024 / P3V<NN>::T) k_pass3v(FftGeo
 constexpr int CP = 16;
 
 // NSC: the product of the radices before (0: known at run time; magic = ceil(2^32 / Ns)).
-template <int RADIX, bool FIRST, bool LAST, int NSC, int SP, class Ld, class St>
+template <int RADIX, bool FIRST, bool LAST, int NSC, int SP, int P, class Ld, class St>
 __device__ __forceinline__ void col_stage(const cx<float>* src, cx<float>* dst, int M, int Ns_, unsigned magic, int twmul,
                                           const cx<float>* __restrict__ tw, Ld ld, St st) {
     const int nbf = M / RADIX, Ns = NSC ? NSC : Ns_;
     const int tmul = nbf / Ns * twmul;   // M / (Ns RADIX) twiddle steps
 #pragma unroll 1
-    for (int b = threadIdx.x; b < nbf * CP; b += blockDim.x) {
-        const int p = b % CP, j = b / CP;
+    for (int b = threadIdx.x; b < nbf * P; b += blockDim.x) {
+        const int p = b % P, j = b / P;
         const int k = Ns == 1 ? 0 : j - Ns * (NSC ? j / NSC : (int)__umulhi((unsigned)j, magic));
         cx<float> v[RADIX];
 #pragma unroll
@@ -825,42 +825,45 @@ __device__ __forceinline__ void col_stage(const cx<float>* src, cx<float>* dst, 
     if (!LAST) __syncthreads();
 }
 
-// Compile-time radix list, from ld to st through the buffers a and b.
-template <int M, int SP, int S, int NS, class Ld, class St>
-__device__ __forceinline__ void col_ct(cx<float>* a, cx<float>* b, int twmul, const cx<float>* tw, Ld ld, St st) {
+// Compile-time radix list, through the buffers a and b.  IO: the first stage loads
+// through ld and the last stores through st; otherwise the lines are in a, and the
+// buffer they end in is returned.
+template <int M, bool IO, int SP, int P, int S, int NS, class Ld, class St>
+__device__ __forceinline__ cx<float>* col_ct(cx<float>* a, cx<float>* b, int twmul, const cx<float>* tw, Ld ld, St st) {
     constexpr RadixList L = radix_list(M);
     if constexpr (S < L.n) {
-        col_stage<L.r[S], S == 0, S == L.n - 1, NS, SP>(a, b, M, NS, 0u, twmul, tw, ld, st);
-        col_ct<M, SP, S + 1, NS * L.r[S]>(b, a, twmul, tw, ld, st);
+        col_stage<L.r[S], IO && S == 0, IO && S == L.n - 1, NS, SP, P>(a, b, M, NS, 0u, twmul, tw, ld, st);
+        return col_ct<M, IO, SP, P, S + 1, NS * L.r[S]>(b, a, twmul, tw, ld, st);
+    } else {
+        return a;
     }
 }
 
-// Run-time radix list (8, 4, 2, 3, 5).  IO: the first stage loads through ld and the last
-// stores through st; otherwise the lines are in a, and the buffer they end in is returned.
-template <bool FIRST, bool LAST, int SP, class Ld, class St>
+// Run-time radix list (8, 4, 2, 3, 5).
+template <bool FIRST, bool LAST, int SP, int P, class Ld, class St>
 __device__ __forceinline__ void col_rt1(int rad, const cx<float>* a, cx<float>* b, int M, int Ns, int twmul,
                                         const cx<float>* tw, Ld ld, St st) {
     const unsigned magic = Ns > 1 ? (unsigned)((0x100000000ull + Ns - 1) / Ns) : 0u;
     switch (rad) {
-        case 8: col_stage<8, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
-        case 4: col_stage<4, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
-        case 2: col_stage<2, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
-        case 3: col_stage<3, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
-        default: col_stage<5, FIRST, LAST, 0, SP>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 8: col_stage<8, FIRST, LAST, 0, SP, P>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 4: col_stage<4, FIRST, LAST, 0, SP, P>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 2: col_stage<2, FIRST, LAST, 0, SP, P>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        case 3: col_stage<3, FIRST, LAST, 0, SP, P>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
+        default: col_stage<5, FIRST, LAST, 0, SP, P>(a, b, M, Ns, magic, twmul, tw, ld, st); break;
     }
 }
-template <bool IO, int SP, class Ld, class St>
+template <bool IO, int SP, int P, class Ld, class St>
 __device__ __forceinline__ cx<float>* col_rt(cx<float>* a, cx<float>* b, int M, const int* rad, int nrad, int twmul,
                                              const cx<float>* tw, Ld ld, St st) {
     if (IO && nrad == 1) {
-        col_rt1<true, true, SP>(rad[0], a, b, M, 1, twmul, tw, ld, st);
+        col_rt1<true, true, SP, P>(rad[0], a, b, M, 1, twmul, tw, ld, st);
         return a;
     }
     int Ns = 1;
     for (int s = 0; s < nrad; ++s) {
-        if (IO && s == 0) col_rt1<true, false, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
-        else if (IO && s == nrad - 1) col_rt1<false, true, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
-        else col_rt1<false, false, SP>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        if (IO && s == 0) col_rt1<true, false, SP, P>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        else if (IO && s == nrad - 1) col_rt1<false, true, SP, P>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
+        else col_rt1<false, false, SP, P>(rad[s], a, b, M, Ns, twmul, tw, ld, st);
         Ns *= rad[s];
         cx<float>* t = a;
         a = b;
@@ -890,8 +893,8 @@ __global__ void __launch_bounds__(256) k_col1(FftGeom g, const cx<float>* __rest
     auto st = [&](int i, int p, cx<float> v) {
         if (kz0 + p < g.nKz) dst[(size_t)i * g.ldz + p] = v;
     };
-    if constexpr (NN > 0) col_ct<NN, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
-    else col_rt<true, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
+    if constexpr (NN > 0) col_ct<NN, true, CP, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
+    else col_rt<true, CP, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
 }
 
 // Pass 2: inverse DFT along y for CP consecutive f_z of one x.
@@ -923,8 +926,8 @@ __global__ void __launch_bounds__(256) k_col2(FftGeom g, const cx<float>* __rest
             m = fmaxf(m, fabsf(v.re) + fabsf(v.im));
         }
     };
-    if constexpr (NN > 0) col_ct<NN, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
-    else col_rt<true, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
+    if constexpr (NN > 0) col_ct<NN, true, CP, CP, 0, 1>(buf + NN * CP, buf, 1, tw, ld, st);   // two stages use buf only
+    else col_rt<true, CP, CP>(buf + N * CP, buf, N, g.rad, g.nrad, 1, tw, ld, st);
     if (fmax2 && fd.out16 >= 0) block_max_to(fmax2 + fd.out16, m);
 }
 
@@ -961,7 +964,7 @@ __global__ void __launch_bounds__(256) k_pass3g(FftGeom g, const cx<float>* __re
     __syncthreads();
     auto none_ld = [](int, int) { return cx<float>{0.f, 0.f}; };
     auto none_st = [](int, int, cx<float>) {};
-    const cx<float>* res = col_rt<false, SP>(buf, buf + M * SP, M, g.rad_h, g.nrad_h, 2, tw, none_ld, none_st);
+    const cx<float>* res = col_rt<false, SP, CP>(buf, buf + M * SP, M, g.rad_h, g.nrad_h, 2, tw, none_ld, none_st);
     float sc = 1.f, s7 = 1.f;   // as in k_pass3v
     if (MODE != P3_FIELD) {
         const float bound = 2.f * (float)nKz * __uint_as_float(fmax2[fd.out16]);
@@ -1200,17 +1203,24 @@ __global__ void k_twiddles(int n, cx<float>* __restrict__ tw) {
 // delta = a g + b applied on load, packed as z_m = d_{2m} + i d_{2m+1}; an
 // M = n/2-point FFT gives Z; X_k = E_k + e^{-2 pi i k/n} O_k with
 // E_k = (Z_k + conj Z_{M-k})/2, O_k = (Z_k - conj Z_{M-k})/(2i), k = 0 .. M.
-template <int P, int NN, bool SQ = false>
-__global__ void __launch_bounds__(NTHR) k_fwd_z(FftGeom g, const float* __restrict__ grid, size_t gstride, float a,
-                                                float b, const cx<float>* __restrict__ twg, cx<float>* __restrict__ T,
-                                                size_t tstride, int msub = 0, int nfull = 0) {
+// Lines side by side as in k_col1 (P consecutive of all n^2; lanes along z for the
+// loads, along k for the stores; 64 lines of 32 points, 16 of 128, so that a stage has
+// work for every thread).  Eight lines on 256 threads before: 512 sub-cubes of 64^3 z
+// 550 -> 377 us, y and x 1 064 -> 349 together (the x pass takes its lines (y, k_z) from
+// one run, so 33 k_z leave no idle lanes there); two grids of 256^3 y and x 224 -> 92.
+template <int NN>
+constexpr int fwd_lines() { return NN == 0 || NN >= 256 ? CP : NN >= 128 ? 32 : 64; }
+
+template <int NN, bool SQ = false>
+__global__ void __launch_bounds__(256) k_fwd_z(FftGeom g, const float* __restrict__ grid, size_t gstride, float a,
+                                               float b, const cx<float>* __restrict__ tw, cx<float>* __restrict__ T,
+                                               size_t tstride, int msub = 0, int nfull = 0) {
+    constexpr int P = fwd_lines<NN>(), SP = P + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int N = NN ? NN : g.n, M = N / 2, H = M + 1;
-    cx<float>* tw = reinterpret_cast<cx<float>*>(smem_raw);
-    cx<float>* buf = tw + N;
-    cx<float>* scr = buf + smem_elems<false, P>(M);
-    const int nyb = (N + P - 1) / P;
-    const int x = blockIdx.x / nyb, y0 = (blockIdx.x % nyb) * P;
+    const int nw = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    const size_t line0 = (size_t)blockIdx.x * P, lines = (size_t)N * N;
     const float* src = grid + (size_t)blockIdx.y * gstride;
     size_t sx = (size_t)N * N, sy = (size_t)N;   // element strides of x and y in the source
     if (msub > 0) {
@@ -1219,69 +1229,109 @@ __global__ void __launch_bounds__(NTHR) k_fwd_z(FftGeom g, const float* __restri
         sy = (size_t)nfull;
         src = grid + (size_t)cx_ * N * sx + (size_t)cy * N * sy + (size_t)cz * N;
     }
-    for (int t = threadIdx.x; t < N; t += NTHR) tw[t] = twg[t];
-    for (int e = threadIdx.x; e < M * P; e += NTHR) {
-        const int m = e % M, p = e / M, y = y0 + p;
-        cx<float> v = {0.f, 0.f};
-        if (y < N) {
-            const float2 r = *reinterpret_cast<const float2*>(src + (size_t)x * sx + (size_t)y * sy + 2 * m);
-            const float r0 = SQ ? r.x * r.x : r.x, r1 = SQ ? r.y * r.y : r.y;
-            v = cx<float>{a * r0 + b, -(a * r1 + b)};   // conjugated
+    for (int p = warp; p < P; p += nw) {
+        const int l = (int)(line0 + p), x = l / N, y = l - x * N;
+        const bool live = line0 + p < lines;
+        const float* row = src + (size_t)x * sx + (size_t)y * sy;
+        for (int m = lane; m < M; m += 32) {
+            cx<float> v = {0.f, 0.f};
+            if (live) {
+                const float2 r = *reinterpret_cast<const float2*>(row + 2 * m);
+                const float r0 = SQ ? r.x * r.x : r.x, r1 = SQ ? r.y * r.y : r.y;
+                v = cx<float>{a * r0 + b, -(a * r1 + b)};   // conjugated
+            }
+            buf[m * SP + p] = v;
         }
-        buf[sidx<false, P>(p, m, M)] = v;
     }
     __syncthreads();
+    auto none_ld = [](int, int) { return cx<float>{0.f, 0.f}; };
+    auto none_st = [](int, int, cx<float>) {};
     const cx<float>* res;
-    if constexpr (NN > 0) res = fft_ct<float, false, P, NN / 2>(buf, scr, tw, 2);
-    else res = fft_pingpong<float, false, P>(buf, scr, M, g.rad_h, g.nrad_h, tw, 2);
-    cx<float>* dst = T + (size_t)blockIdx.y * tstride;
-    for (int e = threadIdx.x; e < H * P; e += NTHR) {
-        const int k = e % H, p = e / H, y = y0 + p;
-        if (y >= N) continue;
-        const cx<float> rk = res[sidx<false, P>(p, k % M, M)], rm = res[sidx<false, P>(p, (M - k) % M, M)];
-        const cx<float> zk = {rk.re, -rk.im}, czm = {rm.re, rm.im};   // Z_k, conj Z_{M-k}
-        const cx<float> E = cscale(cadd(zk, czm), 0.5f);
-        const cx<float> D = cscale(csub(zk, czm), 0.5f);
-        const cx<float> O = {D.im, -D.re};                               // D / i
-        const cx<float> w = {tw[k].re, -tw[k].im};                       // e^{-2 pi i k/n}
-        dst[((size_t)x * N + y) * H + k] = cadd(E, cmul(w, O));
+    if constexpr (NN > 0) res = col_ct<NN / 2, false, SP, P, 0, 1>(buf, buf + M * SP, 2, tw, none_ld, none_st);
+    else res = col_rt<false, SP, CP>(buf, buf + M * SP, M, g.rad_h, g.nrad_h, 2, tw, none_ld, none_st);
+    cx<float>* dst = T + (size_t)blockIdx.y * tstride + line0 * H;
+    for (int p = warp; p < P; p += nw) {
+        if (line0 + p >= lines) break;
+        for (int k = lane; k < H; k += 32) {
+            const cx<float> rk = res[(k == M ? 0 : k) * SP + p], rm = res[(k == 0 ? 0 : M - k) * SP + p];
+            const cx<float> zk = {rk.re, -rk.im}, czm = {rm.re, rm.im};   // Z_k, conj Z_{M-k}
+            const cx<float> E = cscale(cadd(zk, czm), 0.5f);
+            const cx<float> D = cscale(csub(zk, czm), 0.5f);
+            const cx<float> O = {D.im, -D.re};                               // D / i
+            const cx<float> w = {tw[k].re, -tw[k].im};                       // e^{-2 pi i k/n}
+            dst[(size_t)p * H + k] = cadd(E, cmul(w, O));
+        }
     }
 }
 
-// y or x pass, in place: P consecutive k_z of one row o of grid blockIdx.y,
-// element j at o * so + j * sj + k_z.
-template <int P, int NN>
-__global__ void __launch_bounds__(NTHR) k_fwd_axis(FftGeom g, const cx<float>* __restrict__ twg, cx<float>* T,
-                                                   size_t tstride, size_t so, size_t sj) {
+// y or x pass, in place: P consecutive of the L lines of row o of grid blockIdx.y,
+// element j of line l at o * so + j * sj + l (y: the n/2 + 1 lines k_z of one x; x: all
+// the lines (y, k_z)).
+template <int NN, int P>
+__global__ void __launch_bounds__(256) k_fwd_axis(FftGeom g, const cx<float>* __restrict__ tw, cx<float>* T,
+                                                  size_t tstride, size_t so, size_t sj, int L) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int N = NN ? NN : g.n, H = N / 2 + 1;
-    cx<float>* tw = reinterpret_cast<cx<float>*>(smem_raw);
-    cx<float>* buf = tw + N;
-    cx<float>* scr = buf + smem_elems<true, P>(N);
-    const int nkzb = (H + P - 1) / P;
-    const int o = blockIdx.x / nkzb, kz0 = (blockIdx.x % nkzb) * P;
-    cx<float>* t = T + (size_t)blockIdx.y * tstride;
-    for (int q = threadIdx.x; q < N; q += NTHR) tw[q] = twg[q];
-    for (int e = threadIdx.x; e < N * P; e += NTHR) {
-        const int p = e % P, j = e / P, kz = kz0 + p;
+    const int N = NN ? NN : g.n;
+    cx<float>* buf = reinterpret_cast<cx<float>*>(smem_raw);
+    const int nlb = (L + P - 1) / P;
+    const int o = blockIdx.x / nlb, l0 = (blockIdx.x % nlb) * P;
+    cx<float>* t = T + (size_t)blockIdx.y * tstride + (size_t)o * so + l0;
+    auto ld = [&](int i, int p) {
         cx<float> v = {0.f, 0.f};
-        if (kz < H) {
-            const cx<float> u = t[(size_t)o * so + (size_t)j * sj + kz];
+        if (l0 + p < L) {
+            const cx<float> u = t[(size_t)i * sj + p];
             v = cx<float>{u.re, -u.im};
         }
-        buf[sidx<true, P>(p, j, N)] = v;
+        return v;
+    };
+    auto st = [&](int i, int p, cx<float> v) {
+        if (l0 + p < L) t[(size_t)i * sj + p] = cx<float>{v.re, -v.im};
+    };
+    if constexpr (NN > 0) col_ct<NN, true, P, P, 0, 1>(buf + NN * P, buf, 1, tw, ld, st);
+    else col_rt<true, P, P>(buf + N * P, buf, N, g.rad, g.nrad, 1, tw, ld, st);
+}
+
+// y and x passes, P lines a CTA.
+template <int NN, int P>
+cudaError_t launch_fwd_axes(const FftGeom& g, const cx<float>* tw, cx<float>* T, int nb, cudaStream_t st) {
+    const int N = g.n, H = N / 2 + 1;
+    const size_t tstride = (size_t)N * N * H;
+    const int nrad = NN ? radix_list(NN).n : g.nrad, rad0 = NN ? radix_list(NN).r[0] : g.rad[0];
+    const size_t sm = sizeof(cx<float>) * (size_t)N * P * (nrad > 2 ? 2 : 1);   // two stages: one buffer
+    static size_t set = 0;   // raised once per size, never inside a graph capture
+    if (sm > 48 * 1024 && sm > set) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k_fwd_axis<NN, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e != cudaSuccess) return e;
+        set = sm;
     }
-    __syncthreads();
-    const cx<float>* res;
-    if constexpr (NN > 0) res = fft_ct<float, true, P, NN>(buf, scr, tw, 1);
-    else res = fft_pingpong<float, true, P>(buf, scr, N, g.rad, g.nrad, tw, 1);
-    for (int e = threadIdx.x; e < N * P; e += NTHR) {
-        const int p = e % P, j = e / P, kz = kz0 + p;
-        if (kz < H) {
-            const cx<float> r = res[sidx<true, P>(p, j, N)];
-            t[(size_t)o * so + (size_t)j * sj + kz] = cx<float>{r.re, -r.im};
-        }
+    const int t = col_threads(N / rad0 * P);
+    k_fwd_axis<NN, P><<<dim3(N * ((H + P - 1) / P), nb), t, sm, st>>>(g, tw, T, tstride, (size_t)N * H, (size_t)H, H);
+    k_fwd_axis<NN, P><<<dim3((N * H + P - 1) / P, nb), t, sm, st>>>(g, tw, T, tstride, 0, (size_t)N * H, N * H);
+    return cudaGetLastError();
+}
+
+// The three forward passes of nb grids (z with a g + b on load, or of a g^2).
+template <int NN, bool SQ>
+cudaError_t launch_fwd(const FftGeom& g, const float* grid, size_t gstride, float a, float b, const cx<float>* tw,
+                       cx<float>* T, int nb, int msub, int nfull, cudaStream_t st) {
+    constexpr int P = fwd_lines<NN>();
+    const int N = g.n, M = N / 2, H = M + 1;
+    const size_t smz = sizeof(cx<float>) * 2 * (size_t)M * (P + 1);
+    static size_t setz = 0;   // raised once per size, never inside a graph capture
+    cudaError_t e;
+    if (smz > 48 * 1024 && smz > setz) {
+        if ((e = cudaFuncSetAttribute(k_fwd_z<NN, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz)) !=
+            cudaSuccess)
+            return e;
+        setz = smz;
     }
+    const int rz = NN ? radix_list(NN / 2).r[0] : 4;
+    k_fwd_z<NN, SQ><<<dim3((unsigned)(((size_t)N * N + P - 1) / P), nb), col_threads(M / rz * P), smz, st>>>(
+        g, grid, gstride, a, b, tw, T, (size_t)N * N * H, msub, nfull);
+    // 16 lines of more than 896 points and three stages do not fit shared memory twice
+    if (NN == 0 && N > 896) return launch_fwd_axes<NN, NN ? CP : CP / 2>(g, tw, T, nb, st);
+    return launch_fwd_axes<NN, CP>(g, tw, T, nb, st);
 }
 
 // delta(k) = (V/n^3) [X1(k) + e^{-i pi (n_x+n_y+n_z)/n} X2(k)] / (2 W(k)),
@@ -1313,29 +1363,13 @@ __global__ void k_fwd_combine(int N, const cx<float>* __restrict__ T1, const cx<
 template <int NN>
 cudaError_t launch_density_n(const FftGeom& g, const float* pos, long long np, double box, char* ws,
                              cx<float>* out, cudaStream_t st) {
-    constexpr int P = 8;
-    const int N = g.n, M = N / 2, H = M + 1;
+    const int N = g.n, H = N / 2 + 1;
     const DensityLayout L = density_layout(N);
     cx<float>* tw = reinterpret_cast<cx<float>*>(ws + L.tw);
     float* grids = reinterpret_cast<float*>(ws + L.grids);
     cx<float>* T = reinterpret_cast<cx<float>*>(ws + L.spec);
     const size_t gstride = (size_t)N * N * N, tstride = (size_t)N * N * H;
-    const size_t smz = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<false, P>(M));
-    const size_t sma = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<true, P>(N));
-    static size_t setz = 0, seta = 0;   // raised once per size, never inside a graph capture
     cudaError_t e;
-    if (smz > setz) {
-        if ((e = cudaFuncSetAttribute(k_fwd_z<P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz)) !=
-            cudaSuccess)
-            return e;
-        setz = smz;
-    }
-    if (sma > seta) {
-        if ((e = cudaFuncSetAttribute(k_fwd_axis<P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sma)) !=
-            cudaSuccess)
-            return e;
-        seta = sma;
-    }
     if ((e = cudaMemsetAsync(grids, 0, 2 * gstride * sizeof(float), st)) != cudaSuccess) return e;
     k_twiddles<<<(N + 255) / 256, 256, 0, st>>>(N, tw);
     const int cic_blocks = (int)std::min<long long>(4096, (np + 255) / 256);
@@ -1344,10 +1378,7 @@ cudaError_t launch_density_n(const FftGeom& g, const float* pos, long long np, d
     k_cic<<<cic_blocks, 256, 0, st>>>(pos, np, N, scale, sh, sl, grids, grids + gstride);
     // delta_g = count / (N_p / n^3) - 1
     const float a = (float)((double)gstride / (double)np);
-    k_fwd_z<P, NN><<<dim3(N * ((N + P - 1) / P), 2), NTHR, smz, st>>>(g, grids, gstride, a, -1.f, tw, T, tstride);
-    const int nkzb = (H + P - 1) / P;
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, 2), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)N * H, (size_t)H);   // along y
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, 2), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)H, (size_t)N * H);   // along x
+    if ((e = launch_fwd<NN, false>(g, grids, gstride, a, -1.f, tw, T, 2, 0, 0, st)) != cudaSuccess) return e;
     const double V = box * box * box;
     k_fwd_combine<<<4096, 256, 0, st>>>(N, T, T + tstride, (float)(V / (double)gstride), out);
     return cudaGetLastError();
@@ -1395,85 +1426,28 @@ DensityLayout density_layout(int n) {
     return L;
 }
 
-template <int NN>
-cudaError_t launch_forward_square_n(const FftGeom& g, const float* x, float a, const cx<float>* tw, cx<float>* T,
-                                    cudaStream_t st) {
-    constexpr int P = 8;
-    const int N = g.n, M = N / 2, H = M + 1;
-    const size_t smz = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<false, P>(M));
-    const size_t sma = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<true, P>(N));
-    static size_t setz = 0, seta = 0;   // raised once per size, never inside a graph capture
-    cudaError_t e;
-    if (smz > setz) {
-        if ((e = cudaFuncSetAttribute(k_fwd_z<P, NN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smz)) != cudaSuccess)
-            return e;
-        setz = smz;
-    }
-    if (sma > seta) {
-        if ((e = cudaFuncSetAttribute(k_fwd_axis<P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sma)) !=
-            cudaSuccess)
-            return e;
-        seta = sma;
-    }
-    const size_t tstride = (size_t)N * N * H;
-    k_fwd_z<P, NN, true><<<dim3(N * ((N + P - 1) / P), 1), NTHR, smz, st>>>(g, x, 0, a, 0.f, tw, T, tstride);
-    const int nkzb = (H + P - 1) / P;
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, 1), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)N * H, (size_t)H);
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, 1), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)H, (size_t)N * H);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_forward_square(const FftGeom& g, const float* x, float a, const cx<float>* tw, cx<float>* T,
                                   cudaStream_t st) {
     switch (g.n) {
-        case 64: return launch_forward_square_n<64>(g, x, a, tw, T, st);
-        case 96: return launch_forward_square_n<96>(g, x, a, tw, T, st);
-        case 128: return launch_forward_square_n<128>(g, x, a, tw, T, st);
-        case 160: return launch_forward_square_n<160>(g, x, a, tw, T, st);
-        case 256: return launch_forward_square_n<256>(g, x, a, tw, T, st);
-        case 512: return launch_forward_square_n<512>(g, x, a, tw, T, st);
-        default: return launch_forward_square_n<0>(g, x, a, tw, T, st);
+        case 64: return launch_fwd<64, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        case 96: return launch_fwd<96, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        case 128: return launch_fwd<128, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        case 160: return launch_fwd<160, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        case 256: return launch_fwd<256, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        case 512: return launch_fwd<512, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
+        default: return launch_fwd<0, true>(g, x, 0, a, 0.f, tw, T, 1, 0, 0, st);
     }
-}
-
-template <int NN>
-cudaError_t launch_forward_subcubes_n(const FftGeom& g, int nfull, int m, const float* x, float a, cx<float>* tw,
-                                      cx<float>* T, cudaStream_t st) {
-    constexpr int P = 8;
-    const int N = g.n, M = N / 2, H = M + 1, nc = m * m * m;
-    const size_t smz = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<false, P>(M));
-    const size_t sma = sizeof(cx<float>) * ((size_t)N + 2 * (size_t)smem_elems<true, P>(N));
-    static size_t setz = 0, seta = 0;   // raised once per size, never inside a graph capture
-    cudaError_t e;
-    if (smz > setz) {
-        if ((e = cudaFuncSetAttribute(k_fwd_z<P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz)) !=
-            cudaSuccess)
-            return e;
-        setz = smz;
-    }
-    if (sma > seta) {
-        if ((e = cudaFuncSetAttribute(k_fwd_axis<P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sma)) !=
-            cudaSuccess)
-            return e;
-        seta = sma;
-    }
-    const size_t tstride = (size_t)N * N * H;
-    k_twiddles<<<(N + 255) / 256, 256, 0, st>>>(N, tw);
-    k_fwd_z<P, NN><<<dim3(N * ((N + P - 1) / P), nc), NTHR, smz, st>>>(g, x, 0, a, 0.f, tw, T, tstride, m, nfull);
-    const int nkzb = (H + P - 1) / P;
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, nc), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)N * H, (size_t)H);
-    k_fwd_axis<P, NN><<<dim3(N * nkzb, nc), NTHR, sma, st>>>(g, tw, T, tstride, (size_t)H, (size_t)N * H);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_forward_subcubes(const FftGeom& g, int nfull, int m, const float* x, float a, cx<float>* tw,
                                     cx<float>* T, cudaStream_t st) {
     if (m < 1 || m * g.n != nfull || m * m * m > 65535) return cudaErrorInvalidValue;
+    const int nc = m * m * m;
+    k_twiddles<<<(g.n + 255) / 256, 256, 0, st>>>(g.n, tw);
     switch (g.n) {
-        case 64: return launch_forward_subcubes_n<64>(g, nfull, m, x, a, tw, T, st);
-        case 128: return launch_forward_subcubes_n<128>(g, nfull, m, x, a, tw, T, st);
-        default: return launch_forward_subcubes_n<0>(g, nfull, m, x, a, tw, T, st);
+        case 64: return launch_fwd<64, false>(g, x, 0, a, 0.f, tw, T, nc, m, nfull, st);
+        case 128: return launch_fwd<128, false>(g, x, 0, a, 0.f, tw, T, nc, m, nfull, st);
+        default: return launch_fwd<0, false>(g, x, 0, a, 0.f, tw, T, nc, m, nfull, st);
     }
 }
 
