@@ -33,6 +33,15 @@ __device__ __forceinline__ float legendre_w(int ell, int fz2, int n2) {
 
 constexpr int PW_WARPS = 8;   // warps per CTA
 
+// (double)f, from the bits where f is a normal number or zero: the FP64 unit, which
+// also converts, bounds the shell sums of many small spectra (two lanes a clock).
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
+    if (e == 0xFFu || (e == 0u && (u << 1) != 0u)) return (double)f;
+    const uint32_t hi = e == 0u ? u : (u & 0x80000000u) | ((u & 0x7FFFFFFFu) >> 3) + 0x38000000u;
+    return __hiloint2double((int)hi, (int)(u << 29));
+}
+
 // SHOT: also sum w_l per shell (the weights of the shot-noise term); without
 // it those sums stay 0 and the scan carries 4 values instead of 7.
 template <bool SHOT>
@@ -121,10 +130,11 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_power_partial(const cx<float>
             const int snext = __shfl_down_sync(0xffffffffu, s, 1);
             if (s >= 0 && (lane == 31 || snext != s)) {
                 for (int l = 0; l < nell; ++l) {
-                    mine[l * nsh + s] += (double)v[l];
-                    if (SHOT) mine[(nell + l) * nsh + s] += (double)v[4 + l];
+                    mine[l * nsh + s] += widen(v[l]);
+                    if (SHOT) mine[(nell + l) * nsh + s] += widen(v[4 + l]);
                 }
-                mine[2 * nell * nsh + s] += (double)v[3];
+                // the mode count: whole numbers, kept as an integer in the slot
+                reinterpret_cast<long long*>(mine)[2 * nell * nsh + s] += (long long)(int)v[3];
             }
             __syncwarp();
         }
@@ -132,6 +142,12 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_power_partial(const cx<float>
     __syncthreads();
     double* dst = partial + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * per;
     for (int i = threadIdx.x; i < per; i += blockDim.x) {
+        if (i >= 2 * nell * nsh) {   // mode counts
+            long long c = 0;
+            for (int w = 0; w < PW_WARPS; ++w) c += reinterpret_cast<const long long*>(acc)[(size_t)w * per + i];
+            dst[i] = (double)c;
+            continue;
+        }
         double t = 0.0;
         for (int w = 0; w < PW_WARPS; ++w) t += acc[(size_t)w * per + i];   // fixed order
         dst[i] = t;
