@@ -489,6 +489,7 @@ TcSched build_tc_sched(const BinList& bins, const std::vector<int>& out_slots, i
     return h;
 }
 
+constexpr size_t ERR_WORDS = 64;        // one clear takes the error word and the bounds
 constexpr size_t TC_UNIT = 128 * 128;   // FP64 partial values per tensor-core CTA
 
 }  // namespace
@@ -559,8 +560,8 @@ struct bsp_plan {
     TcWork* d_tc_works = nullptr;
     int2* d_tc_pairs = nullptr;
     BinLoc* d_tc_loc = nullptr;
-    int* d_err = nullptr;
-    unsigned* d_fmax = nullptr;   // per-field magnitude bounds for the 16-bit scaling
+    int* d_err = nullptr;         // ERR_WORDS words (the first is the error code), then the bounds
+    unsigned* fmax() const { return reinterpret_cast<unsigned*>(d_err + ERR_WORDS); }   // per-field magnitude bounds for the 16-bit scaling
     int chunk_kb = 1;             // K-blocks (64 points each) per FP32 tensor-memory accumulation
     long long wait_cycles = 0;    // tensor-core pipeline wait limit in clock cycles (0: the kernel's default)
     int tc_max_boxes = 12;        // tensor-core works: at most this many boxes of 8 field rows (N <= 8 x this)
@@ -582,7 +583,6 @@ struct bsp_plan {
         cudaFree(d_fd_delta); cudaFree(d_fd_unit); cudaFree(d_counts);
         cudaFree(d_rep_idx); cudaFree(d_rep_w);
         cudaFree(d_fd_tc); cudaFree(d_tc_works); cudaFree(d_tc_pairs); cudaFree(d_tc_loc); cudaFree(d_err);
-        cudaFree(d_fmax);
         cudaFree(d_tc_units); cudaFree(d_tcu_units);
         cudaFree(d_radial); cudaFree(d_ells); cudaFree(d_tcu_works); cudaFree(d_tcu_pairs); cudaFree(d_tcu_loc);
         u_dev.release();
@@ -819,8 +819,7 @@ bsp_status bsp_plan_create(bsp_plan** out, int n, double box, int n_shells, cons
         (st = upload(&p->d_tw64, tw64)) != BSP_OK || (st = upload(&p->d_fd_delta, fdd)) != BSP_OK ||
         (st = upload(&p->d_fd_unit, fdu)) != BSP_OK || (st = upload(&p->d_fd_tc, fdt)) != BSP_OK ||
         (st = upload(&p->d_fd_raw, std::vector<FieldDesc>{FieldDesc{0, 0, FIELD_RAW, 0, -1, 0, {0, 0}}})) != BSP_OK ||
-        (st = upload(&p->d_err, std::vector<int>{0, 0, 0})) != BSP_OK ||
-        (st = upload(&p->d_fmax, std::vector<unsigned>((size_t)p->nslot() * pad16 + n_shells, 0u))) != BSP_OK) {
+        (st = upload(&p->d_err, std::vector<int>(ERR_WORDS + (size_t)p->nslot() * pad16, 0))) != BSP_OK) {
         delete p;
         return st;
     }
@@ -982,9 +981,8 @@ bsp_status bsp_plan_create_modal(bsp_plan** out, int n, double box, int n_funcs,
     bsp_status st;
     if ((st = upload(&p->d_radial, tab)) != BSP_OK || (st = upload(&p->d_tw32, tw32)) != BSP_OK ||
         (st = upload(&p->d_tw64, tw64)) != BSP_OK || (st = upload(&p->d_fd_delta, fdd)) != BSP_OK ||
-        (st = upload(&p->d_fd_tc, fdt)) != BSP_OK || (st = upload(&p->d_err, std::vector<int>{0, 0, 0})) != BSP_OK ||
-        (st = upload(&p->d_ells, p->ells)) != BSP_OK ||
-        (st = upload(&p->d_fmax, std::vector<unsigned>((size_t)p->nslot() * p->pad16 + 2 * nf, 0u))) != BSP_OK) {
+        (st = upload(&p->d_fd_tc, fdt)) != BSP_OK || (st = upload(&p->d_err, std::vector<int>(ERR_WORDS + (size_t)p->nslot() * p->pad16, 0))) != BSP_OK ||
+        (st = upload(&p->d_ells, p->ells)) != BSP_OK) {
         delete p;
         return st;
     }
@@ -1242,9 +1240,8 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
         cx<float>* t1 = (cx<float>*)(base + L.t1);
         cx<float>* t2 = (cx<float>*)(base + L.t2);
         const int nf = p->nslot() * p->nsh;
-        unsigned* fmax2 = p->d_fmax;              // [slot * pad16 + a]  max |T2| per field (bounds |F|)
-        CK(cudaMemsetAsync(p->d_fmax, 0, sizeof(unsigned) * ((size_t)p->nslot() * p->pad16 + p->nsh), st));
-        CK(cudaMemsetAsync(p->d_err, 0, 3 * sizeof(int), st));   // error code
+        unsigned* fmax2 = p->fmax();              // [slot * pad16 + a]  max |T2| per field (bounds |F|)
+        CK(cudaMemsetAsync(p->d_err, 0, sizeof(int) * (ERR_WORDS + (size_t)p->nslot() * p->pad16), st));   // and the bounds
         if ((ms = clear_tail(p, f0, hi, st)) != BSP_OK) return ms;
         const int f16 = p->prec == BSP_SPLIT_F16 ? 1 : 0;
         for (int f0i = 0; f0i < nf; f0i += p->fb32) {
@@ -1259,7 +1256,6 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
         if ((ms = mark(p, st, 1)) != BSP_OK) return ms;
         double* partial = (double*)(base + L.partial);
         double* tout = (double*)(base + L.tout);
-        CK(cudaMemsetAsync(partial, 0, p->tc_sched.units.size() * TC_UNIT * sizeof(double), st));
         cudaError_t e = launch_contract_tc(f16 != 0, f0, p->kb_rows32, 0, hi, p->groups16, (long long)p->nkb(),
                                            p->d_tc_works, p->d_tc_units,
                                            (int)p->tc_sched.units.size(), p->tc_sched.lsup, p->tc_sched.nsup,
@@ -1387,9 +1383,8 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
         uint32_t* hi = (uint32_t*)(base + L.fields + p->f0_bytes);
         cx<float>* t1 = (cx<float>*)(base + L.t1);
         cx<float>* t2 = (cx<float>*)(base + L.t2);
-        unsigned* fmax2 = p->d_fmax;                    // [slot * pad16 + a] max |T2| per field (bounds |F|)
-        CK(cudaMemsetAsync(p->d_fmax, 0, sizeof(unsigned) * ((size_t)p->nslot() * p->pad16 + 2 * nf), st));
-        CK(cudaMemsetAsync(p->d_err, 0, 3 * sizeof(int), st));   // error code
+        unsigned* fmax2 = p->fmax();                    // [slot * pad16 + a] max |T2| per field (bounds |F|)
+        CK(cudaMemsetAsync(p->d_err, 0, sizeof(int) * (ERR_WORDS + (size_t)p->nslot() * p->pad16), st));   // and the bounds
         if ((ms = clear_tail(p, f0, hi, st)) != BSP_OK) return ms;
         const int f16 = p->prec == BSP_SPLIT_F16 ? 1 : 0;
         for (int fi = 0; fi < nfields; fi += p->fb32) {
@@ -1404,8 +1399,6 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
         if ((ms = mark(p, st, 1)) != BSP_OK) return ms;
         double* part = (double*)(base + L.partial);
         double* upart = (double*)(base + L.partial + p->tc_part_bytes);
-        CK(cudaMemsetAsync(part, 0, p->tc_sched.units.size() * TC_UNIT * sizeof(double), st));
-        if (p->need_u) CK(cudaMemsetAsync(upart, 0, p->tc_u_sched.units.size() * TC_UNIT * sizeof(double), st));
         cudaError_t e = launch_contract_tc(f16 != 0, f0, p->kb_rows32, 0, hi, p->groups16, (long long)p->nkb(),
                                            p->d_tc_works, p->d_tc_units,
                                            (int)p->tc_sched.units.size(), p->tc_sched.lsup, p->tc_sched.nsup,

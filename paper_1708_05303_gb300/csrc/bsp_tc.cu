@@ -249,10 +249,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         S.npc = npc;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // zero every stage once: MMA rows past the tile's groups (N rounds 8 nbox up
-    // to 16) and K-blocks past the end of the grid (no copies) then read zeros
-    for (int i = tid; i < (int)(sizeof(S.f0) + sizeof(S.b)) / 16; i += TC_THREADS)
-        reinterpret_cast<uint4*>(S.f0)[i] = make_uint4(0u, 0u, 0u, 0u);
+    // zero every stage's plane rows once: MMA rows past the tile's groups (N rounds 8 nbox
+    // up to 16) and K-blocks past the end of the grid (no copies) then read zeros
+    for (int t = 0; t < NT; ++t)
+        for (int i = tid; i < (int)N * 16; i += TC_THREADS)   // 16 x 16 bytes a row (hi and lo)
+            reinterpret_cast<uint4*>(S.b[t])[i] = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (tid < TC_M) {
         int2 v = {-1, -1};
@@ -468,13 +469,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         const uint32_t lanebase = tmem + ((uint32_t)(32 * q) << 16);
         const int row = 32 * q + lane;
         const uint32_t c0 = (uint32_t)(EPI_COLS * hc);   // this warp's columns [c0, c0 + 48) within N
-        // the CTA's FP64 slot, [column][pair] (zeroed before the launch): the flushes are
+        // the CTA's FP64 slot, [column][pair]: the first flush stores, the others are
         // fire-and-forget reductions, coalesced over the warp's 32 pairs
         double* dst = partial + (size_t)blockIdx.x * TC_SLOT + row;
         const int pexp = -ilogbf(S.pscale[row]);   // the scales are powers of two
         float sum[EPI_COLS];
 #pragma unroll
         for (int t = 0; t < EPI_COLS; ++t) sum[t] = 0.f;
+        bool first = true;   // no flush yet
         for (int c = 0, g = 0, ce = 0; c < nch; ++c) {
             const int j = c & 1;   // g = c % FL, ce = c % CC
             const bool flush = g == FL - 1 || c == nch - 1;
@@ -525,11 +527,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     const uint32_t col = c0 + (uint32_t)t;
                     if (col < N) {
                         const double v = f32_ldexp_f64(sum[t], pexp + S.fexp[col]);
-                        asm volatile("red.global.add.f64 [%0], %1;" ::"l"(dst + (size_t)col * TC_M), "d"(v)
-                                     : "memory");
+                        if (first) dst[(size_t)col * TC_M] = v;
+                        else
+                            asm volatile("red.global.add.f64 [%0], %1;" ::"l"(dst + (size_t)col * TC_M), "d"(v)
+                                         : "memory");
                     }
                     sum[t] = 0.f;
                 }
+                first = false;
             }
         }
     }
