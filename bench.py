@@ -373,7 +373,7 @@ def main():
         clk = 2070.0
         peak = fp32_peak or N_SM * FP32_LANES_PER_SM * 2 * clk * 1e6 / 1e12
         ach = flop / (con_ms / 1e3) / 1e12
-        roof = {"kernel": "k_contract_cc (FP32 CUDA-core contraction)", "bound": "alu", "achieved": ach,
+        roof = {"kernel": "k_contract_oct (FP32 CUDA-core contraction)", "bound": "alu", "achieved": ach,
                 "peak": peak, "unit": "TFLOP/s", "frac": ach / peak, "traffic": None,
                 "peak_source": ("measured: bsp_fp32_fma_peak (FMA chains, all SMs, CUDA events)" if fp32_peak
                                 else "derived: 152 SMs x 128 FP32 lanes x 2 flop x 2070 MHz"),
@@ -382,9 +382,9 @@ def main():
     elif con_ms >= fft_ms:
         peak = peaks.get("bf16_tflops_sustained", 1700.0)
         # DRAM bytes per launch: ncu capture of this kernel at 160^3 with the same bins,
-        # schedule and default 64-point chunk (11.385 GB read + 0.597 GB written per
+        # schedule and default 64-point chunk (14.231 GB read + 0.602 GB written per
         # launch) scaled by the points
-        traffic = (11.982e9 * (args.n / 160.0) ** 3
+        traffic = (14.833e9 * (args.n / 160.0) ** 3
                    if (args.shells, args.prec, args.chunk) == (64, "split_f16", 0) else None)
         ach = flop / (con_ms / 1e3) / 1e12
         roof = {"kernel": "k_contract_tc (tcgen05 split-product contraction)", "bound": "tensor",
@@ -399,7 +399,7 @@ def main():
         g = fft_alg_bytes(args.n, edges)
         ach = g / (fft_ms / 1e3) / 1e9
         peak = peaks.get("hbm_gbs", 6800.0)
-        roof = {"kernel": "k_pass1/2/3 (filter + inverse FFT)", "bound": "hbm", "achieved": ach, "peak": peak,
+        roof = {"kernel": "filter + inverse FFT passes", "bound": "hbm", "achieved": ach, "peak": peak,
                 "unit": "GB/s", "frac": ach / peak, "traffic": None,
                 "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback 6800 GB/s",
                 "algorithmic": "%.3e bytes per step" % g}

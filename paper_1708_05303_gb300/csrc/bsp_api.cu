@@ -198,7 +198,7 @@ size_t partial_bytes(const HostSched& h, int cols) {
 // FP32 contraction schedule (k_contract_oct).  The pairs (b, c) come in octets
 // (b; c = 8 j .. 8 j + 7); an octet's rows are (l, a) for a in its own a-range.
 // Sorted by the length of that range, the 16 octets of a work waste few rows
-// (32 shells, l = 0, 2, 4: 20 480 multiply-adds per point for 10 872 useful).  All
+// (32 shells, l = 0, 2, 4: 21 504 multiply-adds per point for 10 872 useful).  All
 // warps of a work run the same number of rows: letting each warp have its own put
 // the long ones on one SM partition, and several unrolled variants side by side
 // missed the instruction cache (32 against 21 ms per contraction at 256^3).  A row
@@ -348,11 +348,12 @@ struct TcSched {
 // order at about the same rate and read the same fields while they are in
 // L2.  Nothing holds the CTAs together: a global counter that made every CTA
 // wait for the others at each super-segment (any allowed drift, 1 to 16
-// super-segments) cost 6 % at 512^3 against letting them run (224 -> 210 ms),
+// super-segments) cost 6 % at 512^3 against letting them run (224 -> 210 ms, when a K-block took
+// 1 800 cycles),
 // the acquire load on the contended counter sitting in the copy thread's
 // path.  The cost of a K-block is set by the warps' hand-offs and hardly
-// depends on the MMA N (clock traces on GB300: ~1 700 to 1 800 busy cycles per
-// K-block for N = 32 and N = 96 alike), so the weight is almost flat in N;
+// depends on the MMA N (clock traces on GB300: 1 220 cycles per K-block at
+// N = 32, 1 320 at N = 96), so the weight is almost flat in N;
 // weighting by N, as the first versions did, gave works of small N 1.9x the
 // K-blocks per CTA.  With whole CTAs per work the split is uneven when the
 // works do not divide the SMs (17 works on 152 SMs at 512^3: one work of 8

@@ -17,11 +17,12 @@
 //           -> T1[f_y (compact)][x][f_z]
 //   pass 2: per (x, f_z) pencil, inverse DFT along y -> T2[x][y][f_z]
 //   pass 3: per (x, y) pencil, real inverse DFT along z -> F[x][y][z]
-// Each pass stages a batch of pencils in shared memory, so global reads and
-// writes are contiguous runs; the 1-D transforms are in-place Stockham
-// autosort radix-2/3/4/5/8 stages, ping-ponging between two shared-memory
-// buffers with one barrier per stage.  Twiddles come from a host table of
-// exp(+2 pi i t/N) computed in FP64.
+// Each CTA holds a few lines side by side, so global reads and writes are
+// contiguous runs: n = 512 in registers (k_pass1r, k_pass2r), the z pass of every
+// compile-time size likewise (k_pass3v), the rest as mixed-radix stages through
+// shared memory whose first and last stage touch global memory directly (k_col1,
+// k_col2, k_pass3g).  T1 and T2 rows are padded to 64 bytes.  Twiddles come from a
+// host table of exp(+2 pi i t/N) computed in FP64.
 #include <algorithm>
 #include <type_traits>
 
