@@ -21,7 +21,8 @@
 // contiguous runs: n = 512 in registers (k_pass1r, k_pass2r), the z pass of every
 // compile-time size likewise (k_pass3v), the rest as mixed-radix stages through
 // shared memory whose first and last stage touch global memory directly (k_col1,
-// k_col2, k_pass3g).  T1 and T2 rows are padded to 64 bytes.  Twiddles come from a
+// k_col2, k_pass3g); FP64 (the unit fields of the counts) as Stockham stages on
+// batches of lines (k_pass1, k_pass2, k_pass3).  T1 and T2 rows are padded to 64 bytes.  Twiddles come from a
 // host table of exp(+2 pi i t/N) computed in FP64.
 #include <algorithm>
 #include <type_traits>
