@@ -45,3 +45,19 @@ def test_inverse_transform_sizes(torch_cuda, ora, n):
         bins = [tuple(t) for t in est.bins]
         est.close()
         assert gate(B, ora.bispectrum(dk.astype(np.complex128), n, BOX, edges, bins=bins)["B"]) <= 1e-5
+
+
+# large and small run-time sizes through the three users of the forward passes in turn: one
+# kernel serves them all, and a small size must not take a large one's shared memory away
+def test_run_time_sizes_in_turn(torch_cuda):
+    from paper_1708_05303_gb300 import bsp
+
+    torch = torch_cuda
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    d = torch.randn(400, 400, 201, dtype=torch.complex64, device="cuda", generator=gen)
+    spec = bsp.Spectra(400, BOX, linear_edges(4, 20.0))
+    first = spec.skew(d)[0].cpu()
+    pos = torch.rand(1000, 3, device="cuda", generator=gen) * BOX
+    bsp.density_from_particles(pos, 216, BOX)
+    spec.integrated(d, 2)
+    assert torch.equal(spec.skew(d)[0].cpu(), first)
