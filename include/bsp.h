@@ -191,7 +191,12 @@ bsp_status bsp_modal_project(int n_keep, const double* gamma, int n_rhs, const d
  * bsp_covariance_ws: the same with a device workspace of
  *   bsp_covariance_workspace_size bytes (256-byte aligned; 0: none needed),
  *   through which large matrices are multiplied on the tensor cores as exact
- *   products of integer digits: no less accurate, and many times faster.
+ *   products of integer digits, many times faster.  An entry's error is then one
+ *   rounding (2^-53 of it, and 2^-10 of that) and at most 2^-58 of the product of the two
+ *   columns' largest magnitudes (of value - mean) per row.  Columns whose values lie
+ *   more than 7 bits below their largest on average (outlying rows), that are not
+ *   finite, or whose largest is not within 2^-400 .. 2^400, are multiplied in FP64 as
+ *   by bsp_covariance.
  */
 typedef struct bsp_batch bsp_batch;
 bsp_status bsp_batch_create(bsp_batch** out, int n_sizes, const int* sizes, double box, int n_shells,

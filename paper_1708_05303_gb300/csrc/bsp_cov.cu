@@ -4,21 +4,29 @@
 //
 // Two paths.  The direct one (k_cov) multiplies in FP64; GB300 has two FP64
 // multiply-adds per SM and clock, so 512 x 4 962 values take 11.3 ms there and the
-// unit is the bound.  With a workspace the products run on the tensor cores
-// without losing a bit of what FP64 would keep (the error-free splitting of
-// Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012):
-//   * k_cov_split centres each column, scales it by the power of two above its
-//     largest magnitude, rounds to a 55-bit integer and cuts that into eight
-//     balanced base-128 digits (-64 .. 64), each exact in FP16;
-//   * k_cov_tc forms the products of digits p and q, p + q <= 9, with tcgen05.mma in
-//     FP32 accumulators, one per level p + q.  A level adds at most 8 x 512 products
-//     of at most 2^12, so every partial sum is an integer up to 2^24: exact.
-//     The levels are joined in 64-bit integers and rounded to FP64 once.
-// What is left out is below 2^-54 of the two columns' largest magnitudes per
-// mock, less than the rounding of an FP64 product sum (the measured error against
-// 64 bits is no larger than the direct path's).
-// Columns that are not finite, or so large or small that a product could leave
-// the normal range, are multiplied directly (k_cov_direct).
+// unit is the bound.  With a workspace the products run on the tensor cores (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012):
+//   * k_cov_split centres each column, scales it by the power of two 2^e above its
+//     largest magnitude, rounds to a 63-bit integer and cuts that into eight
+//     balanced base-256 digits (-128 .. 128), each exact in FP16;
+//   * k_cov_tc forms the products of digits p and q, p + q < 8 (from 0), with
+//     tcgen05.mma in FP32 accumulators, one per level p + q.  A level adds at most
+//     8 x 128 products of at most 2^14 between drains, so every partial sum is an
+//     integer up to 2^24: exact.  The levels are joined in 64-bit integers, divided by
+//     M - 1 with a 64-bit reciprocal and rounded to FP64 once.
+// What is lost per mock is at most 9.1 x 2^-64 of 2^(e_i + e_j) (the digit products
+// left out 7.1, the two values' rounding 1 each): below 2^-58 of the product of the two
+// columns' LARGEST magnitudes, whatever the values of that mock.  Where a column's
+// values are mostly far below its largest one (an outlying mock) that could exceed the
+// rounding of an FP64 sum, which is relative to the products themselves; columns whose
+// values lie more than CV_GAP = 7 bits below the largest on (geometric) average are
+// therefore multiplied directly, in k_cov_direct.  Up to there the digits are the more
+// accurate ones entry by entry.  Against exact sums, largest error over the sum of the
+// products' magnitudes, digits and direct: 512 Gaussian mocks 1.0e-16 and 1.7e-15, products of
+// three Gaussians 1.1e-16 and 1.4e-15, two opposite outliers of 2^7 in each of
+// 100 mocks 3.1e-16 and 1.2e-15 (seven-bit digits, before: 4.6e-14; outliers of 2^20: 7e-10,
+// now direct).  So are columns that are not finite, or so large or small that a product
+// could leave the normal range.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -155,7 +163,8 @@ __global__ void __launch_bounds__(256) k_cov_direct(const double* __restrict__ X
 
 constexpr int CV_S = 8;                    // digits
 constexpr int CV_K = 32;                   // mocks per chunk: a 64-byte row of FP16 digits
-constexpr int CV_GROUP = 16;               // chunks (512 mocks) between drains: sums stay below 2^24
+constexpr int CV_GROUP = 4;                // chunks (128 mocks) between drains: sums stay within 2^24
+constexpr int CV_GAP = 7;                  // bits below a column's largest value that its values may lie on average
 constexpr int CV_TM = 128, CV_TN = 64;     // tile (MMA M x N)
 constexpr int CV_EMAX = 400;               // |exponent| of a column that the digits take
 
@@ -163,7 +172,7 @@ constexpr int CV_EMAX = 400;               // |exponent| of a column that the di
 // 16-byte piece c (8 mocks) at piece c ^ ((j >> 1) & 3): the 64-byte swizzle of the
 // tensor-core operand, so that plain copies give the shared-memory image.
 // 1024 threads per 32 columns: sums, then the largest magnitude, then the digits;
-// the strip (256 bytes a mock) is read three times, from L2 after the first.  85 us for
+// the strip (256 bytes a mock) is read three times, from L2 after the first.  89 us for
 // 512 x 4 962 values, set by the FP64 unit (five operations a value) and latency.
 __global__ void __launch_bounds__(1024) k_cov_split(const double* __restrict__ X, int m, int d, int dp, int nkc,
                                                     double* __restrict__ mean, int* __restrict__ ecol,
@@ -195,18 +204,17 @@ __global__ void __launch_bounds__(1024) k_cov_split(const double* __restrict__ X
     __syncthreads();
     if (wid == 0) {
         for (int w = 1; w < 32; ++w) mx = max(mx, (unsigned long long)__double_as_longlong(red[w][lane]));
-        // 2^e above the largest magnitude: |x - mean| 2^(55 - e) < 2^55
+        // 2^e above the largest magnitude: |x - mean| 2^(63 - e) < 2^63 (and 2^10 below it: 53 bits)
         const int ex = (int)(mx >> 52);
         int e = mx == 0 ? 0 : ex - 1022;
         const bool direct = mx != 0 && (ex == 0 || e < -CV_EMAX || e > CV_EMAX);
         if (direct) e = 0;
-        sscale[lane] = direct ? 0.0 : __longlong_as_double((long long)(1023 + 55 - e) << 52);
+        sscale[lane] = direct ? 0.0 : __longlong_as_double((long long)(1023 + 63 - e) << 52);
         ecol[j] = e;
-        const uint32_t bits = __ballot_sync(0xffffffffu, direct || !live);
-        if (lane == 0) dmask[blockIdx.x] = bits;
     }
     __syncthreads();
     const double sc = sscale[lane];
+    int gap = 0, cnt = 0;   // bits that the values lie below the largest (up to 63), and how many are not 0
     for (int o = wid; o < nkc * (CV_K / 8); o += 32) {   // eight mocks of one column
         uint32_t q[CV_S][4];
 #pragma unroll
@@ -215,15 +223,23 @@ __global__ void __launch_bounds__(1024) k_cov_split(const double* __restrict__ X
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int k = o * 8 + 2 * k2 + u;
-                v[u] = live && k < m && sc != 0.0 ? __double2ll_rn((x[(size_t)k * d] - mu) * sc) : 0ll;
+                v[u] = 0;
+                if (live && k < m && sc != 0.0) {
+                    const double y = x[(size_t)k * d] - mu;
+                    v[u] = __double2ll_rn(y * sc);
+                    if (v[u] != 0 || (__double_as_longlong(y) << 1) != 0) {
+                        gap += min(63, __clzll(llabs(v[u])) - 1);
+                        ++cnt;
+                    }
+                }
             }
 #pragma unroll
             for (int t = CV_S - 1; t >= 0; --t) {   // balanced digits, the lowest first; what is left is the top one
                 int g[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    g[u] = t == 0 ? (int)v[u] : (int)((v[u] + 64) & 127) - 64;
-                    v[u] = (v[u] - g[u]) >> 7;
+                    g[u] = t == 0 ? (int)v[u] : (int)((v[u] + 128) & 255) - 128;
+                    v[u] = (v[u] - g[u]) >> 8;
                 }
                 asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(q[t][k2]) : "f"((float)g[1]), "f"((float)g[0]));
             }
@@ -233,6 +249,17 @@ __global__ void __launch_bounds__(1024) k_cov_split(const double* __restrict__ X
         for (int t = 0; t < CV_S; ++t)
             digits[((size_t)(kc * CV_S + t) * dp + j) * 4 + (c ^ ((j >> 1) & 3))] =
                 make_uint4(q[t][0], q[t][1], q[t][2], q[t][3]);
+    }
+    red[wid][lane] = __hiloint2double(gap, cnt);   // the bits (red was last read before the barrier above)
+    __syncthreads();
+    if (wid == 0) {
+        for (int w = 1; w < 32; ++w) {
+            gap += __double2hiint(red[w][lane]);
+            cnt += __double2loint(red[w][lane]);
+        }
+        const bool direct = sc == 0.0 || gap > (long long)CV_GAP * cnt;
+        const uint32_t bits = __ballot_sync(0xffffffffu, direct || !live);
+        if (lane == 0) dmask[blockIdx.x] = bits;
     }
 }
 
@@ -257,36 +284,48 @@ __device__ __forceinline__ void mma_ss(uint32_t d, uint64_t a, uint64_t b, uint3
         : "memory");
 }
 
-// (hi 2^28 + lo) 2^e rounded to FP64 (nearest, ties to even); the result is a normal number or 0.
-__device__ __forceinline__ double join_round(long long hi, long long lo, int e) {
-    __int128 t = ((__int128)hi << 28) + lo;
+// 1 / (M - 1) as rec 2^-(63 + sh), rec in [2^63, 2^64).
+struct CvRecip {
+    unsigned long long rec;
+    int sh;
+};
+CvRecip cov_recip(int m) {
+    const unsigned long long q = (unsigned long long)m - 1;
+    int sh = 0;
+    while ((1ull << sh) < q) ++sh;
+    return CvRecip{(unsigned long long)(((unsigned __int128)1 << (63 + sh)) / q), sh};
+}
+
+// (hi 2^32 + lo) 2^e / (M - 1) rounded to FP64 (nearest; the quotient is truncated to
+// 63 bits or more before, 2^-10 of a last place); the result is a normal number or 0.
+__device__ __forceinline__ double join_round(long long hi, long long lo, int e, CvRecip r) {
+    const __int128 t = ((__int128)hi << 32) + lo;
     if (t == 0) return 0.0;
     const unsigned long long sign = t < 0 ? 0x8000000000000000ull : 0ull;
     const unsigned __int128 u = t < 0 ? (unsigned __int128)(-t) : (unsigned __int128)t;
     const unsigned long long uh = (unsigned long long)(u >> 64), ul = (unsigned long long)u;
-    const int n = uh ? 127 - __clzll((long long)uh) : 63 - __clzll((long long)ul);   // top bit
-    unsigned long long q;
-    if (n <= 52) {
-        q = ul << (52 - n);
-    } else {
-        const int s = n - 52;   // 1 .. 40
-        q = (unsigned long long)(u >> s);
-        const unsigned long long rem = ul & ((1ull << s) - 1), half = 1ull << (s - 1);
-        if (rem > half || (rem == half && (q & 1))) ++q;
-    }
+    const int n = uh ? 127 - __clzll((long long)uh) : 63 - __clzll((long long)ul);   // top bit, up to 95
+    const unsigned long long top = n > 63 ? (unsigned long long)(u >> (n - 63)) : ul << (63 - n);
+    unsigned long long p = __umul64hi(top, r.rec);   // [2^62, 2^64): the value is p 2^(n - 62 - sh + e)
+    const int s = (int)(~p >> 63);
+    p <<= s;
+    const unsigned long long rem = p & 2047;
+    unsigned long long q = p >> 11;
+    if (rem > 1024 || (rem == 1024 && (q & 1))) ++q;
     // q in [2^52, 2^53]: a carry out of the mantissa moves into the exponent
-    return __longlong_as_double((long long)(sign | (((unsigned long long)(n + e + 1022) << 52) + q)));
+    return __longlong_as_double((long long)(sign | (((unsigned long long)(n + e - r.sh - s + 1023) << 52) + q)));
 }
 
 // One 128 x 64 tile per CTA: eight levels of 64 columns fill tensor memory, so A and B
 // both come from shared memory, 96 KB for 32 mocks, two stages.  The MMAs read 6 KB
-// of shared memory per 32 cycles of tensor work, which bounds them at 48; 580 us for
-// 1 560 tiles of 512 mocks (52 us a tile, 27 us of that the MMAs' operand reads).
+// of shared memory per 32 cycles of tensor work, which bounds them at 48; 572 us for
+// 1 560 tiles of 512 mocks (52 us a tile, 27 us of that the MMAs' operand reads and four
+// drains of ~2 us, which nothing overlaps).
 constexpr int CV_THREADS = 320;   // warp 0 copies, warp 1 MMAs, warps 2 .. 9 drain (quadrant warp % 4, 32 columns each)
 
 __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restrict__ digits, int dp, int nkc,
                                                           const int* __restrict__ ecol,
-                                                          const uint32_t* __restrict__ dmask, int m, int d,
+                                                          const uint32_t* __restrict__ dmask, CvRecip recip, int d,
                                                           double* __restrict__ C) {
     extern __shared__ uint8_t cv_raw[];
     CvSmem& S = *reinterpret_cast<CvSmem*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
@@ -379,7 +418,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
     } else {
         const int c0 = 32 * ((warp - 2) >> 2);
         const uint32_t lanebase = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + c0;
-        long long hi[32], lo[32];   // levels 2 .. 5 and 6 .. 9, in units of 2^-33 and 2^-61
+        long long hi[32], lo[32];   // levels 0 .. 3 and 4 .. 7, in units of 2^-38 and 2^-70
 #pragma unroll
         for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
         const int ng = (nkc + CV_GROUP - 1) / CV_GROUP;
@@ -407,8 +446,8 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
                     int v[CV_S];
 #pragma unroll
                     for (int t = 0; t < CV_S; ++t) v[t] = __float2int_rn(__uint_as_float(r[t][u]));
-                    hi[c + u] += ((((((long long)v[0] << 7) + v[1]) << 7) + v[2]) << 7) + v[3];
-                    lo[c + u] += ((((((long long)v[4] << 7) + v[5]) << 7) + v[6]) << 7) + v[7];
+                    hi[c + u] += ((((((long long)v[0] << 8) + v[1]) << 8) + v[2]) << 8) + v[3];
+                    lo[c + u] += ((((((long long)v[4] << 8) + v[5]) << 8) + v[6]) << 8) + v[7];
                 }
             }
             tc_fence_before();
@@ -416,7 +455,6 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
             if (lane == 0) mbar_arrive(&S.acc_empty);
         }
         const int i = I * CV_TM + 32 * (warp & 3) + lane;
-        const double inv = 1.0 / (double)(m - 1);
         const int ei = ecol[i];
         const uint32_t di = dmask[i >> 5] >> lane & 1u, dj = dmask[(J * CV_TN + c0) >> 5];   // direct (or past d)
         const bool bad = S.abort != 0;   // a wait gave up: no number
@@ -426,7 +464,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
             const int j = J * CV_TN + c0 + c;
             double v = 0.0;
             if (!di && !(dj >> c & 1u) && j >= i) {
-                v = bad ? __longlong_as_double(0x7ff8000000000000ll) : join_round(hi[c], lo[c], ei + ecol[j] - 61) * inv;
+                v = bad ? __longlong_as_double(0x7ff8000000000000ll) : join_round(hi[c], lo[c], ei + ecol[j] - 70, recip);
                 C[(size_t)j * d + i] = v;   // lanes: consecutive i
             }
             stage[lane * 33 + c] = v;
@@ -510,7 +548,7 @@ bsp_status bsp_covariance_ws(int m, int d, const double* rows, double* mean, dou
     int tiles = 0;
     for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
     k_cov_split<<<L.dp / 32, 1024, 0, st>>>(rows, m, d, L.dp, L.nkc, mean, ecol, dmask, (uint4*)digits);
-    k_cov_tc<<<tiles, CV_THREADS, smem, st>>>(digits, L.dp, L.nkc, ecol, dmask, m, d, cov);
+    k_cov_tc<<<tiles, CV_THREADS, smem, st>>>(digits, L.dp, L.nkc, ecol, dmask, cov_recip(m), d, cov);
     const long long nb = (d + 31) / 32;
     k_cov_direct<<<(int)std::min<long long>(nb * nb, 152 * 8), 256, 0, st>>>(rows, mean, m, d, dmask, cov);
     cudaError_t e = cudaGetLastError();
