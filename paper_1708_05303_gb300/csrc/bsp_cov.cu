@@ -326,7 +326,7 @@ constexpr int CV_THREADS = 320;   // warp 0 copies, warp 1 MMAs, warps 2 .. 9 dr
 __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restrict__ digits, int dp, int nkc,
                                                           const int* __restrict__ ecol,
                                                           const uint32_t* __restrict__ dmask, CvRecip recip, int d,
-                                                          double* __restrict__ C) {
+                                                          double* __restrict__ C, long long wlim) {
     extern __shared__ uint8_t cv_raw[];
     CvSmem& S = *reinterpret_cast<CvSmem*>((reinterpret_cast<uintptr_t>(cv_raw) + 1023) & ~(uintptr_t)1023);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
             int issued = 0;
             for (int k = 0; k < nkc && !S.abort; ++k) {
                 const int s = k & 1, u = k >> 1;
-                if (u > 0 && !mbar_wait(&S.empty[s], (u - 1) & 1)) {
+                if (u > 0 && !mbar_wait(&S.empty[s], (u - 1) & 1, wlim)) {
                     S.abort = 1;
                     break;
                 }
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
                 }
                 issued = k + 1;
             }
-            for (int k = max(0, issued - 2); k < issued; ++k)   // copies in flight land before the CTA ends
+            for (int k = max(0, issued - 2); k < issued; ++k)   // copies in flight land before the CTA ends (the long limit)
                 if (!mbar_wait(&S.full[k & 1], (k >> 1) & 1)) S.abort = 1;
         }
     } else if (warp == 1) {
@@ -389,13 +389,12 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
         int done = 0;
         for (int k = 0; k < nkc; ++k) {
             const int s = k & 1, g = k / CV_GROUP, kg = k % CV_GROUP;
-            bool ok = kg != 0 || g == 0 || mbar_wait(&S.acc_empty, (g - 1) & 1);
-            ok = ok && mbar_wait(&S.full[s], (k >> 1) & 1);
-            if (!__all_sync(0xffffffffu, ok)) {
+            // the chunk's copies, and where it starts a group the accumulators read out: one barrier per lane
+            const bool acc = kg == 0 && g > 0 && (lane & 1);
+            if (!warp_wait<128>(smem_u32(acc ? &S.acc_empty : &S.full[s]), (uint32_t)((acc ? g - 1 : k >> 1) & 1), wlim, &S.abort)) {
                 S.abort = 1;
                 break;
             }
-            if (__shfl_sync(0xffffffffu, S.abort, 0)) break;
             tc_fence_after();
             if (elect_one()) {
                 const uint64_t a0 = sw64_desc(smem_u32(S.a[s][0])), b0 = sw64_desc(smem_u32(S.b[s][0]));
@@ -422,9 +421,12 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
 #pragma unroll
         for (int c = 0; c < 32; ++c) hi[c] = lo[c] = 0;
         const int ng = (nkc + CV_GROUP - 1) / CV_GROUP;
-        for (int g = 0; g < ng && !S.abort; ++g) {
-            if (!mbar_wait(&S.acc_full, g & 1)) {
+        // the whole warp waits and decides together: the loads of tensor memory below are .aligned
+        bool bad = false;   // a wait gave up: no numbers
+        for (int g = 0; g < ng; ++g) {
+            if (!warp_wait<1>(smem_u32(&S.acc_full), (uint32_t)(g & 1), wlim, &S.abort)) {
                 S.abort = 1;
+                bad = true;
                 break;
             }
             tc_fence_after();
@@ -457,22 +459,29 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
         const int i = I * CV_TM + 32 * (warp & 3) + lane;
         const int ei = ecol[i];
         const uint32_t di = dmask[i >> 5] >> lane & 1u, dj = dmask[(J * CV_TN + c0) >> 5];   // direct (or past d)
-        const bool bad = S.abort != 0;   // a wait gave up: no number
-        double* stage = reinterpret_cast<double*>(S.a[0]) + (size_t)(warp - 2) * (32 * 33);   // the operands are used up
+        if (!bad) {
+            double* stage = reinterpret_cast<double*>(S.a[0]) + (size_t)(warp - 2) * (32 * 33);   // the operands are used up
 #pragma unroll
-        for (int c = 0; c < 32; ++c) {
-            const int j = J * CV_TN + c0 + c;
-            double v = 0.0;
-            if (!di && !(dj >> c & 1u) && j >= i) {
-                v = bad ? __longlong_as_double(0x7ff8000000000000ll) : join_round(hi[c], lo[c], ei + ecol[j] - 70, recip);
-                C[(size_t)j * d + i] = v;   // lanes: consecutive i
+            for (int c = 0; c < 32; ++c) {
+                const int j = J * CV_TN + c0 + c;
+                double v = 0.0;
+                if (!di && !(dj >> c & 1u) && j >= i) {
+                    v = join_round(hi[c], lo[c], ei + ecol[j] - 70, recip);
+                    C[(size_t)j * d + i] = v;   // lanes: consecutive i
+                }
+                stage[lane * 33 + c] = v;
             }
-            stage[lane * 33 + c] = v;
-        }
-        __syncwarp();
-        for (int r = 0; r < 32; ++r) {      // lanes: consecutive j
-            const int ir = I * CV_TM + 32 * (warp & 3) + r, j = J * CV_TN + c0 + lane;
-            if (!(__shfl_sync(0xffffffffu, di, r) | (dj >> lane & 1u)) && j > ir) C[(size_t)ir * d + j] = stage[r * 33 + lane];
+            __syncwarp();
+            for (int r = 0; r < 32; ++r) {      // lanes: consecutive j
+                const int ir = I * CV_TM + 32 * (warp & 3) + r, j = J * CV_TN + c0 + lane;
+                if (!(__shfl_sync(0xffffffffu, di, r) | (dj >> lane & 1u)) && j > ir) C[(size_t)ir * d + j] = stage[r * 33 + lane];
+            }
+        } else {   // (copies may still land in shared memory: nothing passes through it)
+            for (int c = 0; c < 32; ++c) {
+                const int j = J * CV_TN + c0 + c;
+                if (di || (dj >> c & 1u) || j < i) continue;
+                C[(size_t)j * d + i] = C[(size_t)i * d + j] = __longlong_as_double(0x7ff8000000000000ll);
+            }
         }
     }
     tc_fence_before();
@@ -503,6 +512,31 @@ CovLayout cov_layout(int m, int d) {
 // 747 against 99; 512 x 4 962: 11 329 against 662).
 bool cov_use_tc(int m, int d) { return m >= 100 || (double)m * d * d >= 1.0e7; }
 
+// The digits' path; wlim: limit of the pipeline's waits in clock cycles (an entry of a tile
+// whose wait runs out is NaN).
+cudaError_t launch_cov_digits(int m, int d, const double* rows, double* mean, double* cov, void* ws, long long wlim,
+                              cudaStream_t st) {
+    const CovLayout L = cov_layout(m, d);
+    int* ecol = (int*)ws;
+    uint32_t* dmask = (uint32_t*)((char*)ws + L.mask);
+    uint8_t* digits = (uint8_t*)ws + L.digits;
+    const size_t smem = sizeof(CvSmem) + 1024;
+    static bool attr = false;   // once, never inside a graph capture
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_cov_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        attr = true;
+    }
+    const int nJ = (d + CV_TN - 1) / CV_TN, nI = (d + CV_TM - 1) / CV_TM;
+    int tiles = 0;
+    for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
+    k_cov_split<<<L.dp / 32, 1024, 0, st>>>(rows, m, d, L.dp, L.nkc, mean, ecol, dmask, (uint4*)digits);
+    k_cov_tc<<<tiles, CV_THREADS, smem, st>>>(digits, L.dp, L.nkc, ecol, dmask, cov_recip(m), d, cov, wlim);
+    const long long nb = (d + 31) / 32;
+    k_cov_direct<<<(int)std::min<long long>(nb * nb, 152 * 8), 256, 0, st>>>(rows, mean, m, d, dmask, cov);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 }  // namespace bsp
@@ -531,27 +565,8 @@ bsp_status bsp_covariance_ws(int m, int d, const double* rows, double* mean, dou
     if (m < 2 || d < 1 || !rows || !mean || !cov) return BSP_EINVAL;
     if (!cov_use_tc(m, d)) return bsp_covariance(m, d, rows, mean, cov, stream);
     if (!ws || ((uintptr_t)ws & 255u)) return BSP_EINVAL;
-    const CovLayout L = cov_layout(m, d);
-    if (ws_bytes < L.end) return BSP_ENOMEM;
-    cudaStream_t st = (cudaStream_t)stream;
-    int* ecol = (int*)ws;
-    uint32_t* dmask = (uint32_t*)((char*)ws + L.mask);
-    uint8_t* digits = (uint8_t*)ws + L.digits;
-    const size_t smem = sizeof(CvSmem) + 1024;
-    static bool attr = false;   // once, never inside a graph capture
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_cov_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return record_cuda_error(e, "covariance");
-        attr = true;
-    }
-    const int nJ = (d + CV_TN - 1) / CV_TN, nI = (d + CV_TM - 1) / CV_TM;
-    int tiles = 0;
-    for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;
-    k_cov_split<<<L.dp / 32, 1024, 0, st>>>(rows, m, d, L.dp, L.nkc, mean, ecol, dmask, (uint4*)digits);
-    k_cov_tc<<<tiles, CV_THREADS, smem, st>>>(digits, L.dp, L.nkc, ecol, dmask, cov_recip(m), d, cov);
-    const long long nb = (d + 31) / 32;
-    k_cov_direct<<<(int)std::min<long long>(nb * nb, 152 * 8), 256, 0, st>>>(rows, mean, m, d, dmask, cov);
-    cudaError_t e = cudaGetLastError();
+    if (ws_bytes < cov_layout(m, d).end) return BSP_ENOMEM;
+    const cudaError_t e = launch_cov_digits(m, d, rows, mean, cov, ws, WAIT_CYCLES, (cudaStream_t)stream);
     return e == cudaSuccess ? BSP_OK : record_cuda_error(e, "covariance");
 }
 
