@@ -443,13 +443,10 @@ cudaError_t launch_contract_oct(const float* rows, const float* px, const float*
     const int nrow = max_a + (sym ? 2 : 1) * max_x;
     const uint32_t stage_bytes = (uint32_t)nrow * OCT_RB;
     const size_t smem = 2 * (size_t)stage_bytes + (size_t)nrow * sizeof(float*);
-    static bool attr[2] = {false, false};
+    static SmemLimit limit[2];
     auto kern = sym ? k_contract_oct<true> : k_contract_oct<false>;
-    if (!attr[sym != 0]) {   // once per variant, never inside a graph capture
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, OCT_SMEM_MAX);
-        if (e != cudaSuccess) return e;
-        attr[sym != 0] = true;
-    }
+    const cudaError_t e = raise_smem(limit[sym != 0], OCT_SMEM_MAX, kern);
+    if (e != cudaSuccess) return e;
     kern<<<dim3(nwork, nsplit), OCT_THREADS, smem, st>>>(rows, px, py, fstride, works, stage, stage_bytes, npts, seg,
                                                          partial);
     return cudaGetLastError();

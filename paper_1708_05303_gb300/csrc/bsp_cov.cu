@@ -521,12 +521,9 @@ cudaError_t launch_cov_digits(int m, int d, const double* rows, double* mean, do
     uint32_t* dmask = (uint32_t*)((char*)ws + L.mask);
     uint8_t* digits = (uint8_t*)ws + L.digits;
     const size_t smem = sizeof(CvSmem) + 1024;
-    static bool attr = false;   // once, never inside a graph capture
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_cov_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = raise_smem(limit, smem, k_cov_tc);
+    if (e != cudaSuccess) return e;
     const int nJ = (d + CV_TN - 1) / CV_TN, nI = (d + CV_TM - 1) / CV_TM;
     int tiles = 0;
     for (int I = 0; I < nI; ++I) tiles += nJ - 2 * I;

@@ -1008,19 +1008,11 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
     const size_t t1_stride = (size_t)g.nK * N * g.ldz, t2_stride = (size_t)N * N * g.ldz;
     const size_t sm12 = sizeof(cx<double>) * ((size_t)N + 2 * (size_t)smem_elems<true, P>(N));
     const size_t sm3 = sizeof(cx<double>) * ((size_t)N + 2 * (size_t)smem_elems<false, P3>(M));
-    // raise the dynamic shared-memory limit once per size (never inside a graph capture)
-    static size_t set = 0;
-    if (std::max(sm12, sm3) > set) {
-        cudaError_t e;
-        if ((e = cudaFuncSetAttribute(k_pass1<double, P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm12)) !=
-                cudaSuccess ||
-            (e = cudaFuncSetAttribute(k_pass2<double, P, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm12)) !=
-                cudaSuccess ||
-            (e = cudaFuncSetAttribute(k_pass3<double, P3, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3)) !=
-                cudaSuccess)
-            return e;
-        set = std::max(sm12, sm3);
-    }
+    static SmemLimit limit12, limit3;
+    cudaError_t e;
+    if ((e = raise_smem(limit12, sm12, k_pass1<double, P, NN>, k_pass2<double, P, NN>)) != cudaSuccess ||
+        (e = raise_smem(limit3, sm3, k_pass3<double, P3, NN>)) != cudaSuccess)
+        return e;
     const int nkzb = (g.nKz + P - 1) / P;
     k_pass1<double, P, NN><<<dim3(g.nK * nkzb, nfields), NTHR, sm12, st>>>(g, delta, shell_of, radial, d_fields, tw, t1,
                                                                            t1_stride);
@@ -1043,15 +1035,8 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
     const size_t t1_stride = (size_t)g.nK * N * g.ldz, t2_stride = (size_t)N * N * g.ldz;
     cudaError_t e;
     if constexpr (NN == 512) {
-        static bool set = false;   // never inside a graph capture
-        if (!set) {
-            if ((e = cudaFuncSetAttribute(k_pass1r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2r_smem_bytes())) !=
-                    cudaSuccess ||
-                (e = cudaFuncSetAttribute(k_pass2r, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p2r_smem_bytes())) !=
-                    cudaSuccess)
-                return e;
-            set = true;
-        }
+        static SmemLimit limit;
+        if ((e = raise_smem(limit, p2r_smem_bytes(), k_pass1r, k_pass2r)) != cudaSuccess) return e;
         const int nkzb = (g.nKz + P2R - 1) / P2R;
         k_pass1r<<<dim3(g.nK * nkzb, nfields), NTHR, p2r_smem_bytes(), st>>>(g, delta, shell_of, radial, d_fields, tw, t1,
                                                                              t1_stride);
@@ -1060,13 +1045,8 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
     } else {
         const int nrad = NN ? radix_list(NN).n : g.nrad, rad0 = NN ? radix_list(NN).r[0] : g.rad[0];
         const size_t sm = sizeof(cx<float>) * (size_t)N * CP * (nrad > 2 ? 2 : 1);   // two stages: one buffer
-        static size_t set = 0;
-        if (sm > 48 * 1024 && sm > set) {
-            if ((e = cudaFuncSetAttribute(k_col1<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess ||
-                (e = cudaFuncSetAttribute(k_col2<NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-                return e;
-            set = sm;
-        }
+        static SmemLimit limit;
+        if ((e = raise_smem(limit, sm, k_col1<NN>, k_col2<NN>)) != cudaSuccess) return e;
         const int nkzb = (g.nKz + CP - 1) / CP, thr = col_threads(N / rad0 * CP);
         k_col1<NN><<<dim3(g.nK * nkzb, nfields), thr, sm, st>>>(g, delta, shell_of, radial, d_fields, tw, t1, t1_stride);
         k_col2<NN><<<dim3(N * nkzb, nfields), thr, sm, st>>>(g, t1, t1_stride, tw, t2, t2_stride, d_fields, fmax2);
@@ -1080,13 +1060,8 @@ cudaError_t launch_n(const FftGeom& g, const cx<float>* delta, const int16_t* sh
     } else {
         auto kern = !kbm ? k_pass3g<P3_FIELD> : f16 ? k_pass3g<P3_F16> : k_pass3g<P3_BF16>;
         const size_t sm = sizeof(cx<float>) * 2 * (size_t)M * (CP + 1);
-        static size_t set[3] = {0, 0, 0};
-        const int ki = !kbm ? 0 : f16 ? 1 : 2;
-        if (sm > 48 * 1024 && sm > set[ki]) {
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm)) != cudaSuccess)
-                return e;
-            set[ki] = sm;
-        }
+        static SmemLimit limit[3];
+        if ((e = raise_smem(limit[!kbm ? 0 : f16 ? 1 : 2], sm, kern)) != cudaSuccess) return e;
         kern<<<dim3((unsigned)(((size_t)N * N + CP - 1) / CP), nfields), col_threads(M * CP / 4), sm, st>>>(
             g, t2, t2_stride, tw, d_fields, out, out_stride, hi, lo != nullptr, fmax2, lay);
     }
@@ -1300,13 +1275,9 @@ cudaError_t launch_fwd_axes(const FftGeom& g, const cx<float>* tw, cx<float>* T,
     const size_t tstride = (size_t)N * N * H;
     const int nrad = NN ? radix_list(NN).n : g.nrad, rad0 = NN ? radix_list(NN).r[0] : g.rad[0];
     const size_t sm = sizeof(cx<float>) * (size_t)N * P * (nrad > 2 ? 2 : 1);   // two stages: one buffer
-    static size_t set = 0;   // raised once per size, never inside a graph capture
-    if (sm > 48 * 1024 && sm > set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_fwd_axis<NN, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e != cudaSuccess) return e;
-        set = sm;
-    }
+    static SmemLimit limit;
+    const cudaError_t e = raise_smem(limit, sm, k_fwd_axis<NN, P>);
+    if (e != cudaSuccess) return e;
     const int t = col_threads(N / rad0 * P);
     k_fwd_axis<NN, P><<<dim3(N * ((H + P - 1) / P), nb), t, sm, st>>>(g, tw, T, tstride, (size_t)N * H, (size_t)H, H);
     k_fwd_axis<NN, P><<<dim3((N * H + P - 1) / P, nb), t, sm, st>>>(g, tw, T, tstride, 0, (size_t)N * H, N * H);
@@ -1320,14 +1291,9 @@ cudaError_t launch_fwd(const FftGeom& g, const float* grid, size_t gstride, floa
     constexpr int P = fwd_lines<NN>();
     const int N = g.n, M = N / 2, H = M + 1;
     const size_t smz = sizeof(cx<float>) * 2 * (size_t)M * (P + 1);
-    static size_t setz = 0;   // raised once per size, never inside a graph capture
-    cudaError_t e;
-    if (smz > 48 * 1024 && smz > setz) {
-        if ((e = cudaFuncSetAttribute(k_fwd_z<NN, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smz)) !=
-            cudaSuccess)
-            return e;
-        setz = smz;
-    }
+    static SmemLimit limitz;
+    const cudaError_t e = raise_smem(limitz, smz, k_fwd_z<NN, SQ>);
+    if (e != cudaSuccess) return e;
     const int rz = NN ? radix_list(NN / 2).r[0] : 4;
     k_fwd_z<NN, SQ><<<dim3((unsigned)(((size_t)N * N + P - 1) / P), nb), col_threads(M / rz * P), smz, st>>>(
         g, grid, gstride, a, b, tw, T, (size_t)N * N * H, msub, nfull);

@@ -7,12 +7,30 @@
 #include <stdint.h>
 
 #include "../../include/bsp.h"
+#include "bsp_smem.h"
 
 namespace bsp {
 
 // Record `where: <CUDA error text>` as this thread's bsp_last_error() and
 // return BSP_ECUDA (defined in bsp_api.cu).
 bsp_status record_cuda_error(cudaError_t e, const char* where);
+
+// Give the kernels at least `bytes` of dynamic shared memory on the current device (only
+// where they need more than the 48 KB that every kernel has; a first call sets an
+// attribute, so the library's callers make it outside graph capture).
+template <class... K>
+cudaError_t raise_smem(SmemLimit& limit, size_t bytes, K*... kernels) {
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    return limit.raise<cudaError_t>(dev, bytes, [&](size_t b) {
+        cudaError_t r = cudaSuccess;
+        for (const void* k : {(const void*)kernels...})
+            if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)b);
+        return r;
+    });
+}
 
 template <typename R>
 struct __align__(2 * sizeof(R)) cx {

@@ -208,13 +208,9 @@ cudaError_t launch_power(const cx<float>* delta, const cx<float>* Q, double num_
     if (smem > 227 * 1024) return cudaErrorInvalidValue;
     const bool shot = nbar > 0.0;
     auto kern = shot ? k_power_partial<true> : k_power_partial<false>;
-    static size_t set[2] = {0, 0};   // raised once per size and variant, never inside a graph capture
-    cudaError_t e;
-    if (smem > 48 * 1024 && smem > set[shot]) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        set[shot] = smem;
-    }
+    static SmemLimit limit[2];
+    const cudaError_t e = raise_smem(limit[shot], smem, kern);
+    if (e != cudaSuccess) return e;
     if (nbatch < 1 || nbatch > 65535 || (nbatch > 1 && Q)) return cudaErrorInvalidValue;
     kern<<<dim3(nblocks, nbatch), 32 * PW_WARPS, smem, st>>>(delta, Q, g, shell_of, nsh, ells, partial, bstride,
                                                              dc_weight, n2top);

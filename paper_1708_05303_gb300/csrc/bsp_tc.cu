@@ -558,15 +558,10 @@ cudaError_t launch_contract_tc(bool f16, const float* f0, int f0_rows, int f0_ro
                                cudaStream_t st, long long wait_cycles) {
     const size_t smem = tc_smem_bytes();
     const long long wlim = wait_cycles > 0 ? wait_cycles : WAIT_CYCLES;
-    static bool set16 = false, setb = false;   // once per kernel, never inside a graph capture
+    static SmemLimit limit[2];
     auto kern = f16 ? k_contract_tc<true> : k_contract_tc<false>;
-    cudaError_t e;
-    bool& set = f16 ? set16 : setb;
-    if (!set) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        set = true;
-    }
+    const cudaError_t e = raise_smem(limit[f16], smem, kern);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nunits);
     cfg.blockDim = dim3(TC_THREADS);
