@@ -415,13 +415,18 @@ class Batch:
         import torch
 
         m, d = rows.shape
-        mean = torch.empty(d, dtype=torch.float64, device="cuda")
-        cov = torch.empty((d, d), dtype=torch.float64, device="cuda")
         nb = ctypes.c_size_t()
         _check(load().bsp_covariance_workspace_size(int(m), int(d), ctypes.byref(nb)), "bsp_covariance")
-        ws = torch.empty(max(nb.value, 256), dtype=torch.uint8, device="cuda")
+        # from the pool of the stream that writes them: memory just freed on the current
+        # stream may still be in use there
+        here = torch.cuda.current_stream()
+        with torch.cuda.stream(stream):
+            mean = torch.empty(d, dtype=torch.float64, device="cuda")
+            cov = torch.empty((d, d), dtype=torch.float64, device="cuda")
+            ws = torch.empty(max(nb.value, 256), dtype=torch.uint8, device="cuda")
         if stream is not None:
-            ws.record_stream(stream)   # released here, in use there
+            for t in (mean, cov):
+                t.record_stream(here)   # read there once the caller has waited, and perhaps released first
         _check(load().bsp_covariance_ws(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _dptr(ws), int(nb.value),
                                         _stream_handle(stream)), "bsp_covariance")
         return mean, cov
