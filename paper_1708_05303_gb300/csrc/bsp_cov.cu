@@ -509,8 +509,15 @@ CovLayout cov_layout(int m, int d) {
 // The tensor-core path from where it is the faster one.  The direct one takes 0.36 us
 // per mock where its tiles fit the SMs at once (100 x 50 values: 47 us on both; 160 x
 // 128: 66 against 50) and m d^2 / 1.1e6 us beyond (64 x 400: 51 against 39; 512 x 1 000:
-// 747 against 99; 512 x 4 962: 11 329 against 662).
-bool cov_use_tc(int m, int d) { return m >= 100 || (double)m * d * d >= 1.0e7; }
+// 747 against 99; 512 x 4 962: 11 329 against 666).  Not where few columns, padded to 128, would
+// take far more digits than the matrix itself (16 x 128 bytes a mock; up to 1 GiB is let pass:
+// 400 000 x 3 values), nor past 2^22 mocks, up to which the 64-bit level sums hold
+// (2^40.4 a mock).
+bool cov_use_tc(int m, int d) {
+    if (m > (1 << 22) || !(m >= 100 || (double)m * d * d >= 1.0e7)) return false;
+    const CovLayout L = cov_layout(m, d);
+    return L.end <= (size_t)1 << 30 || L.dp <= 4ll * d;
+}
 
 // The digits' path; wlim: limit of the pipeline's waits in clock cycles (an entry of a tile
 // whose wait runs out is NaN).
