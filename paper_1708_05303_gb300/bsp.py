@@ -423,12 +423,19 @@ class Batch:
         with torch.cuda.stream(stream):
             mean = torch.empty(d, dtype=torch.float64, device="cuda")
             cov = torch.empty((d, d), dtype=torch.float64, device="cuda")
-            ws = torch.empty(max(nb.value, 256), dtype=torch.uint8, device="cuda")
+            try:
+                ws = torch.empty(nb.value, dtype=torch.uint8, device="cuda") if nb.value else None
+            except torch.cuda.OutOfMemoryError:
+                ws = None                # no room for the digits: the direct path needs none
         if stream is not None:
             for t in (mean, cov):
                 t.record_stream(here)   # read there once the caller has waited, and perhaps released first
-        _check(load().bsp_covariance_ws(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _dptr(ws), int(nb.value),
-                                        _stream_handle(stream)), "bsp_covariance")
+        if ws is None:
+            _check(load().bsp_covariance(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _stream_handle(stream)),
+                   "bsp_covariance")
+        else:
+            _check(load().bsp_covariance_ws(int(m), int(d), _dptr(rows), _dptr(mean), _dptr(cov), _dptr(ws), int(nb.value),
+                                            _stream_handle(stream)), "bsp_covariance")
         return mean, cov
 
     def close(self):
