@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "bsp_cic.h"
 #include "bsp_internal.h"
 
 namespace bsp {
@@ -1149,15 +1150,8 @@ __global__ void k_cic(const float* __restrict__ pos, long long np, int n, double
                 t2[a] = t;
             } else {
 #pragma unroll
-                for (int gs = 0; gs < 2; ++gs) {
-                    double u = (double)p * scale - 0.5 * gs;
-                    u -= floor(u / n) * n;   // into [0, n)
-                    int bi = (int)floor(u);
-                    if (bi >= n) bi -= n;
-                    if (bi < 0) bi += n;
-                    (gs ? b2 : b1)[a] = bi;
-                    (gs ? t2 : t1)[a] = (float)(u - (double)bi);
-                }
+                for (int gs = 0; gs < 2; ++gs)
+                    cic_wrap((double)p * scale - 0.5 * gs, n, (gs ? b2 : b1)[a], (gs ? t2 : t1)[a]);
             }
         }
         cic_deposit(g1, n, b1, t1);
