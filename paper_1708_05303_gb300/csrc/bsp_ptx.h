@@ -79,7 +79,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, long lon
 // one after another, three barriers that had long completed took 250 cycles each.
 // The first SPIN tests poll, the rest sleep (a sleeping wait wakes some 300 cycles
 // late: starting with one cost the contraction 20 %, even when the phase was complete).
-// False once `limit` cycles have passed or *abort is set.
+// The same result in every lane: false once `limit` cycles have passed or *abort is set.
 template <int SPIN>
 __device__ __forceinline__ bool warp_wait(uint32_t addr, uint32_t parity, long long limit, const volatile int* abort) {
     bool done = mbar_test(addr, parity);
@@ -98,20 +98,21 @@ __device__ __forceinline__ bool warp_wait(uint32_t addr, uint32_t parity, long l
     }
     const bool sleep = limit >= (1ll << 20);
     const long long t0 = clock64();
+    // every lane tests again, also those whose phase is complete: with the sleeping test under a
+    // branch (or a predicate) of `done`, a warp with one open barrier came apart here and its other lanes
+    // left with true (tests/gpu_probes/warp_wait.cu); testing again costs nothing measurable
     while (true) {
-        if (!done) {
-            if (sleep) {
-                uint32_t d;
-                asm volatile(
-                    "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-                    " selp.u32 %0, 1, 0, p;\n}\n"
-                    : "=r"(d)
-                    : "r"(addr), "r"(parity), "r"(2000u)
-                    : "memory");
-                done = d != 0;
-            } else {
-                done = mbar_test(addr, parity);
-            }
+        if (sleep) {
+            uint32_t d;
+            asm volatile(
+                "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+                " selp.u32 %0, 1, 0, p;\n}\n"
+                : "=r"(d)
+                : "r"(addr), "r"(parity), "r"(2000u)
+                : "memory");
+            done = d != 0;
+        } else {
+            done = mbar_test(addr, parity);
         }
         if (__all_sync(0xffffffffu, done)) {
             __syncwarp();
