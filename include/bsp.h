@@ -438,8 +438,9 @@ bsp_status bsp_set_wait_limit(bsp_plan* plan, long long cycles);
 
 /*
  * Error word of the plan's kernels: 0 if no kernel has reported a problem,
- * else a bit mask of bounded waits that gave up (the kernel then stopped
- * early, released its tensor memory and left its outputs undefined).
+ * else a bit mask of the bounded waits that gave up first, over all thread blocks (the
+ * waits they stopped are not in it; the kernel then ended early, released its
+ * tensor memory and left its outputs undefined).
  * Synchronous (waits for the device).  Returns BSP_ETIMEOUT if nonzero.
  */
 bsp_status bsp_device_status(bsp_plan* plan, int* code);

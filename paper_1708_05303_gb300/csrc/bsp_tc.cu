@@ -196,7 +196,11 @@ __device__ __forceinline__ double f32_ldexp_f64(float f, int k) {
     return __longlong_as_double((long long)b);
 }
 
+// A wait gave up.  Where another one of the CTA had done so before, this one was stopped by it
+// and is no finding of its own: only the first is recorded.  (Told apart here: a warp_wait with a third
+// result cost 2 % on its hot path.)
 __device__ __forceinline__ void set_abort(TcSmem& S, int* err, int code) {
+    if (S.abort) return;
     S.abort = 1;
     atomicOr(err, code);
 }
@@ -250,7 +254,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     // zero every stage's plane rows once: MMA rows past the tile's groups (N rounds 8 nbox
-    // up to 16) and K-blocks past the end of the grid (no copies) then read zeros
+    // up to 16) then read zeros.  (K-blocks past the end of the grid have no copies and may read
+    // an earlier K-block's planes: their pair products are zeros.)
     for (int t = 0; t < NT; ++t)
         for (int i = tid; i < (int)N * 16; i += TC_THREADS)   // 16 x 16 bytes a row (hi and lo)
             reinterpret_cast<uint4*>(S.b[t])[i] = make_uint4(0u, 0u, 0u, 0u);
