@@ -430,7 +430,7 @@ bsp_status bsp_set_accumulation_chunk(bsp_plan* plan, int points);
  * (2^33 cycles, about 4 s).  A wait that runs out makes the kernel record
  * the error in the plan's error word (bsp_device_status), stop issuing work,
  * wait for its own copies and MMAs in flight (always with the default limit)
- * and release its tensor memory; the call's outputs are then undefined.
+ * and release its tensor memory; the call's outputs are then NaN.
  * For failure-path testing: a limit of a few hundred cycles makes the first
  * wait for a copy run out.  1 <= cycles <= 2^40, or 0.
  */
@@ -439,8 +439,8 @@ bsp_status bsp_set_wait_limit(bsp_plan* plan, long long cycles);
 /*
  * Error word of the plan's kernels: 0 if no kernel has reported a problem,
  * else a bit mask of the bounded waits that gave up first, over all thread blocks (the
- * waits they stopped are not in it; the kernel then ended early, released its
- * tensor memory and left its outputs undefined).
+ * waits they stopped are not in it; the kernel then ended early and released its
+ * tensor memory, and the call's outputs are NaN).
  * Synchronous (waits for the device).  Returns BSP_ETIMEOUT if nonzero.
  */
 bsp_status bsp_device_status(bsp_plan* plan, int* code);

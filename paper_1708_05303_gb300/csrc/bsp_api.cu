@@ -1266,7 +1266,7 @@ static bsp_status compute_impl(bsp_plan* p, const void* delta_k, double nbar, vo
         if ((ms = mark(p, st, 2)) != BSP_OK) return ms;
         const double V = p->box * p->box * p->box;
         e = launch_reduce(partial, 0, TC_UNIT, 128, p->d_tc_loc, (int)p->tc_sched.loc.size(),
-                          (int)p->bins.size(), p->d_counts, 1.0 / (V * (double)p->npts()), 1, tout, B, st);
+                          (int)p->bins.size(), p->d_counts, 1.0 / (V * (double)p->npts()), 1, tout, B, st, nullptr, p->d_err);
         if (e != cudaSuccess) return cuda_fail(e, "reduce");
         if ((ms = mark(p, st, 3)) != BSP_OK) return ms;
         p->launches_last = launches + 2;
@@ -1418,10 +1418,10 @@ bsp_status bsp_modal_compute(bsp_plan* p, const void* delta_k, void* ws, void* s
         }
         if ((ms = mark(p, st, 2)) != BSP_OK) return ms;
         e = launch_reduce(part, 0, TC_UNIT, 128, p->d_tc_loc, (int)p->tc_sched.loc.size(),
-                          (int)nall, p->d_counts, 1.0, 2, nullptr, tfull, st);
+                          (int)nall, p->d_counts, 1.0, 2, nullptr, tfull, st, nullptr, p->d_err);
         if (e == cudaSuccess && p->need_u)
             e = launch_reduce(upart, 0, TC_UNIT, 128, p->d_tcu_loc,
-                              (int)p->tc_u_sched.loc.size(), (int)nall, p->d_counts, 1.0, 2, nullptr, ufull, st);
+                              (int)p->tc_u_sched.loc.size(), (int)nall, p->d_counts, 1.0, 2, nullptr, ufull, st, nullptr, p->d_err);
         if (e != cudaSuccess) return cuda_fail(e, "reduce (modal)");
         launches += p->need_u ? 2 : 1;
     }

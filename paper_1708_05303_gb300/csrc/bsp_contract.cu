@@ -362,10 +362,12 @@ constexpr int RED_WARPS = 8;
 __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce(
     const double* __restrict__ partial, int nsplit, size_t unit, int row_stride, const BinLoc* __restrict__ loc,
     int nout, int nbins, const double* __restrict__ counts, double scale, int mode, double* __restrict__ T_out,
-    double* __restrict__ out, ShotTerms shot) {
+    double* __restrict__ out, ShotTerms shot, const int* __restrict__ err) {
     __shared__ double red[4][RED_WARPS][32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, i = blockIdx.x * 32 + lane;
     const int nset = 1 + shot.n;
+    // the contraction's error word: after a wait that gave up, slots may hold an earlier call's sums
+    const bool gave_up = err != nullptr && *err != 0;
     if (i < nout) {
         const BinLoc L = loc[i];
         // nsplit > 0: slots work*nsplit .. +nsplit; else slots L.work .. L.work + L.pad
@@ -386,6 +388,7 @@ __global__ void __launch_bounds__(32 * RED_WARPS) k_reduce(
         u[t] = red[t][0][lane];
         for (int k = 1; k < RED_WARPS; ++k) u[t] += red[t][k][lane];
     }
+    if (gave_up) u[0] = __longlong_as_double(0x7ff8000000000000ll);
     if (T_out) T_out[i] = u[0];
     if (mode == 0) {
         out[i] = rint(u[0] * scale);
@@ -454,14 +457,14 @@ cudaError_t launch_contract_oct(const float* rows, const float* px, const float*
 
 cudaError_t launch_reduce(const double* partial, int nsplit, size_t unit, int row_stride, const BinLoc* loc,
                           int nout, int nbins, const double* counts, double scale, int mode, double* T_out,
-                          double* out, cudaStream_t st, const ShotTerms* shot) {
+                          double* out, cudaStream_t st, const ShotTerms* shot, const int* err) {
     ShotTerms none{};
     none.n = 0;
     if (nout <= 0) return cudaSuccess;
     if (unit == 0) unit = CC_OUT;
     if (row_stride == 0) row_stride = CC_COLS;
     k_reduce<<<(nout + 31) / 32, 32 * RED_WARPS, 0, st>>>(partial, nsplit, unit, row_stride, loc, nout, nbins, counts, scale,
-                                                 mode, T_out, out, shot ? *shot : none);
+                                                          mode, T_out, out, shot ? *shot : none, err);
     return cudaGetLastError();
 }
 

@@ -185,7 +185,7 @@ cudaError_t launch_gather_reps(const double* fields, size_t npts, int nsh, const
 cudaError_t launch_reduce(const double* partial, int nsplit, size_t unit, int row_stride,
                           const BinLoc* loc, int nout, int nbins, const double* counts, double scale,
                           int mode, double* T_out, double* out, cudaStream_t st,
-                          const ShotTerms* shot = nullptr);
+                          const ShotTerms* shot = nullptr, const int* err = nullptr);
 
 // ---- launchers (bsp_tc.cu) ----
 // Operands in the K-block-major layout (FieldLayout): F0 row of shell s in
