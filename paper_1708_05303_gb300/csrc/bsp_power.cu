@@ -133,8 +133,9 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_power_partial(const cx<float>
                     mine[l * nsh + s] += widen(v[l]);
                     if (SHOT) mine[(nell + l) * nsh + s] += widen(v[4 + l]);
                 }
-                // the mode count: whole numbers, kept as an integer in the slot
-                reinterpret_cast<long long*>(mine)[2 * nell * nsh + s] += (long long)(int)v[3];
+                // the mode count: whole numbers, kept as the bits of an integer in the slot
+                double& count = mine[2 * nell * nsh + s];
+                count = __longlong_as_double(__double_as_longlong(count) + (long long)(int)v[3]);
             }
             __syncwarp();
         }
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(32 * PW_WARPS) k_power_partial(const cx<float>
     for (int i = threadIdx.x; i < per; i += blockDim.x) {
         if (i >= 2 * nell * nsh) {   // mode counts
             long long c = 0;
-            for (int w = 0; w < PW_WARPS; ++w) c += reinterpret_cast<const long long*>(acc)[(size_t)w * per + i];
+            for (int w = 0; w < PW_WARPS; ++w) c += __double_as_longlong(acc[(size_t)w * per + i]);
             dst[i] = (double)c;
             continue;
         }
