@@ -381,10 +381,10 @@ def main():
                 "issued_frac": (issued / (con_ms / 1e3) / 1e12) / peak}
     elif con_ms >= fft_ms:
         peak = peaks.get("bf16_tflops_sustained", 1700.0)
-        # DRAM bytes per launch: ncu capture of this kernel at 160^3 with the same bins,
-        # schedule and default 64-point chunk (14.231 GB read + 0.602 GB written per
-        # launch) scaled by the points
-        traffic = (14.833e9 * (args.n / 160.0) ** 3
+        # DRAM bytes per launch: ncu capture of this kernel at 512^3 (684.1 GB read + 19.8 GB
+        # written), scaled by the points for other grids with the same bins, schedule and
+        # default 64-point chunk (160^3 reads less per point: more of it stays in L2)
+        traffic = (703.97e9 * (args.n / 512.0) ** 3
                    if (args.shells, args.prec, args.chunk) == (64, "split_f16", 0) else None)
         ach = flop / (con_ms / 1e3) / 1e12
         roof = {"kernel": "k_contract_tc (tcgen05 split-product contraction)", "bound": "tensor",

@@ -648,8 +648,8 @@ __global__ void __launch_bounds__(NTHR) k_pass3(FftGeom g, const cx<R>* __restri
 // radix-16 stage.  Fields and time before -> now: 288 FP32 fields of 256^3 14.2 ->
 // 4.9 ms (4.4 at the copy rate), 72 of 160^3 1.33 -> 0.27 ms, 150 operand sets of 256^3
 // 8.9 -> 4.0 ms, 96 of 512^3 (16 x 16 in registers before, staged for 16-byte stores)
-// 20.5 -> 18.8 ms.  Bound at 512^3: L1 wavefronts, 76 % busy (T2 rows of 1 040 bytes, the
-// 4-byte plane stores).
+// 20.5 -> 18.8 ms.  Bound for FP32 fields of 256^3: L1, 77 % busy, then DRAM at 77 % of the
+// copy rate (36 fields 533 us); the planes of 512^3 are written at 67 % of it.
 template <int NN>
 struct P3V {
     static constexpr int M = NN / 2;
@@ -793,8 +793,8 @@ __global__ void __launch_bounds__(P3V<NN>::T, 1024 / P3V<NN>::T) k_pass3v(FftGeo
 // lines (no conflicts, no index division), and a stage has (length / radix) CP
 // butterflies for the CTA's threads.  Passes 1 and 2 take their first stage straight
 // from global memory and store the last one there, in runs of CP consecutive f_z
-// (128 bytes, in rows padded to 64).  Bound by latency: two to four stages with a barrier
-// each on 2 to 12 warps a CTA.  Eight lines on 256 threads with run-time divisions in
+// (128 bytes, in rows padded to 64).  Bound by issue slots and latency: at 150^3 pass 2 has 64 %
+// of its slots busy, pass 3 78 %; two to four stages with a barrier each.  Eight lines on 256 threads with run-time divisions in
 // every index, before, left most threads idle.  Before -> now, microseconds: 42 fields
 // of 150^3 pass 1 107 -> 70, 2 302 -> 190, 3 1 331 -> 630; 150 of 256^3 pass 2 3 159 -> 2 000;
 // 72 of 160^3 pass 2 160 -> 130; 32^3 with 8 shells, all three 50 -> 30.
@@ -1112,7 +1112,7 @@ __device__ __forceinline__ void cic_deposit(float* g, int n, const int (&b)[3], 
 // (j + 1/2) H).  Cell units u = p n / box to ~2^-46 as an FP32 pair (p times the pair
 // sh + sl), far below the 2^-25 to which the weights round their fraction; positions
 // outside [0, box) take FP64 and the wrap.  4 Mi particles on 256^3: 172 us, bound by the
-// L2's additions, 4 to 8 a particle and grid (FP64 with two divisions a coordinate and
+// way of the reductions, 4 to 8 a particle and grid, through L1 (77 % busy) and L2 (60 %) (FP64 with two divisions a coordinate and
 // 16 scalar additions a particle: 722 us).
 __global__ void k_cic(const float* __restrict__ pos, long long np, int n, double scale, float sh, float sl,
                       float* __restrict__ g1, float* __restrict__ g2) {
