@@ -413,7 +413,8 @@ __global__ void __launch_bounds__(CV_THREADS, 1) k_cov_tc(const uint8_t* __restr
             __syncwarp();
             done = k + 1;
         }
-        if (done > 0 && !__all_sync(0xffffffffu, mbar_wait(&S.empty[(done - 1) & 1], ((done - 1) >> 1) & 1))) S.abort = 1;
+        // the last MMAs finish before tensor memory is released (the long limit)
+        if (done > 0 && !warp_wait<1>(smem_u32(&S.empty[(done - 1) & 1]), (uint32_t)(((done - 1) >> 1) & 1), WAIT_CYCLES, nullptr)) S.abort = 1;
     } else {
         const int c0 = 32 * ((warp - 2) >> 2);
         const uint32_t lanebase = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + c0;

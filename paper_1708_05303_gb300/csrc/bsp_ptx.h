@@ -79,7 +79,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, long lon
 // one after another, three barriers that had long completed took 250 cycles each.
 // The first SPIN tests poll, the rest sleep (a sleeping wait wakes some 300 cycles
 // late: starting with one cost the contraction 20 %, even when the phase was complete).
-// The same result in every lane: false once `limit` cycles have passed or *abort is set.
+// The same result in every lane: false once `limit` cycles have passed or *abort is set
+// (abort may be null: a last wait that nothing else ends).
 template <int SPIN>
 __device__ __forceinline__ bool warp_wait(uint32_t addr, uint32_t parity, long long limit, const volatile int* abort) {
     bool done = mbar_test(addr, parity);
@@ -118,7 +119,7 @@ __device__ __forceinline__ bool warp_wait(uint32_t addr, uint32_t parity, long l
             __syncwarp();
             return true;
         }
-        if (__any_sync(0xffffffffu, *abort != 0 || clock64() - t0 > limit)) return false;
+        if (__any_sync(0xffffffffu, (abort != nullptr && *abort != 0) || clock64() - t0 > limit)) return false;
     }
 }
 

@@ -397,7 +397,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             done = k + 1;
         }
         // the last MMAs must finish before tensor memory is released (long limit)
-        if (done > 0 && !__all_sync(0xffffffffu, mbar_wait(&S.kb_done[(done - 1) % NT], ((done - 1) / NT) & 1)) && lane == 0)
+        if (done > 0 && !warp_wait<1>(smem_u32(&S.kb_done[(done - 1) % NT]), (uint32_t)(((done - 1) / NT) & 1), WAIT_CYCLES, nullptr) &&
+            lane == 0)
             atomicOr(err, 32);
     } else if (warp >= W_PRO0 && warp < W_PRO0 + N_PRO) {
         // lane quadrant q of tensor memory = pairs 32 q .. 32 q + 31; part t of each
